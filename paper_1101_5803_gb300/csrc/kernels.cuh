@@ -104,6 +104,7 @@ struct CglsArgs {
     const float2* spec32;   // PSF spectra of the FFT problems, [n_probs][spec_stride] (FP32 contexts)
     const double2* spec64;  // the same in FP64
     long long spec_stride;  // elements per problem
+    int max_smem;           // dynamic shared memory a CTA may take (cluster kernel)
 };
 
 // ---------------------------------------------------------------------------

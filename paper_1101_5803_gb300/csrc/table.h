@@ -27,6 +27,9 @@ struct KernelTable {
     const void* fwdb[MAX_K];
     const void* pixmap;  // pixel-ordered ray map for the banded forward batch
     const void* psf_spectra[2];  // PSF spectra of the FFT-convolution problems
+    // cluster[K][nt]: general kernel on a thread-block cluster (FP32), nt = 0
+    // for 256 threads a CTA, 1 for 512
+    const void* cluster[MAX_K][2];
 };
 
 void fill_f32_k5(KernelTable& t);
@@ -40,5 +43,10 @@ void fill_f64(KernelTable& t);
 void fill_fast(KernelTable& t);
 void fill_iter(KernelTable& t);
 void fill_fwd_band(KernelTable& t);
+void fill_cluster_a(KernelTable& t);
+void fill_cluster_b(KernelTable& t);
+void fill_cluster_c(KernelTable& t);
+void fill_cluster_d(KernelTable& t);
+void fill_cluster_e(KernelTable& t);
 
 }  // namespace mirage
