@@ -33,169 +33,65 @@ int mlp_fail(int code, const std::string& msg) {
         if (e_ != cudaSuccess) return mlp_fail(MIRAGE_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// C[M x N] (FP32, row-major, ldc) = sum_k A(m, k) B(k, n) with
-//   A(m, k) = A[m * sam + k * sak],  B(k, n) = B[k * sbk + n * sbn]  (BF16)
-// on the fifth-generation tensor cores: one CTA of four warps per 128 x BN
-// output tile, accumulator in tensor memory (BN FP32 columns), K in chunks
-// of TC_BK staged by the CTA into shared memory as K-major core matrices
-// (8 rows x 8 BF16), TC_BK / 16 tcgen05.mma of K = 16 per chunk issued by one
-// thread, completion through an mbarrier.  Edges are zero-filled.  Should a
+// A layer's products on the fifth-generation tensor cores,
+//   C[M x N] = sum_k A(m, k) B(k, n),
+//   A(m, k) = A[m * sam + k * sak],  B(k, n) = B[k * sbk + n * sbn]  (BF16),
+// with what follows them (bias, activation, loss gradient) applied to the
+// accumulator before it leaves the CTA.
+//
+// What bounds the network is latency: a training step of the 7-256-256-256-2
+// network on 256 rows is 0.2 GFLOP, and 27 launches of products, activations
+// and sums took 194 us of it.  So a layer is one launch (its dW, db and dA
+// together, which are independent), and a product one pass: a CTA of eight
+// warps per 128 x BN tile loads up to TC_BK = 256 of K at once (every load in
+// flight together), stages it as K-major core matrices (8 rows x 8 BF16),
+// issues all its tcgen05.mma (K = 16 each, in order of k, so that an element
+// is the same sum whatever the chunk) from one thread and waits once.  The
+// core matrices lie TC_LBO bytes apart along K and TC_SBO along M and N, padded
+// so that neither the row-wise stores nor the transposed ones (8 x 8 blocks
+// turned in registers) meet in a bank.  Edges are zero-filled.  Should a
 // completion wait run out (about a second), the tile is written as NaN.
-constexpr int TC_BM = 128, TC_BK = 64;
+constexpr int TC_BM = 128, TC_BK = 256, TC_T = 256;
+constexpr int TC_LBO = 144, TC_SBO = TC_BK / 8 * TC_LBO + 16;
 
 template <int BN>
 constexpr int tc_smem_bytes() {
-    return (TC_BM + BN) * TC_BK * 2 + 16;
+    return (TC_BM + BN) / 8 * TC_SBO + 16;
 }
+// byte offset of core-matrix row r (16 bytes: k-octet o)
+__device__ __forceinline__ int tc_row(int r, int o) { return (r >> 3) * TC_SBO + o * TC_LBO + (r & 7) * 16; }
 
-// element (r, k) of a staged tile -> core matrix (r / 8, k / 8), k-chunks
-// innermost: BF16 index ((r / 8) * TC_KO + k / 8) * 64 + (r % 8) * 8 + k % 8, so
-// one 16-byte row of a core matrix holds 8 consecutive k of one row r
-constexpr int TC_KO = TC_BK / 8;  // k-octets (core-matrix columns) per staged row group
-__device__ __forceinline__ int tc_at(int r, int k) { return ((r >> 3) * TC_KO + (k >> 3)) * 64 + (r & 7) * 8 + (k & 7); }
+enum : int { EPI_PLAIN = 0, EPI_HIDDEN = 1, EPI_OUT = 2, EPI_BACK = 3 };
 
-// How an operand view is staged: rows contiguous along k (16-byte rows of
-// 8 k), a transposed view (8 rows contiguous at one k), or element by element
-enum : int { ST_KROW = 0, ST_KCOL = 1, ST_SCALAR = 2 };
-
-__device__ __forceinline__ int stage_mode(const __nv_bfloat16* src, long s_row, long s_k) {
-    const bool al = ((uintptr_t)src & 15) == 0;
-    if (s_k == 1 && (s_row & 7) == 0 && al) return ST_KROW;
-    if (s_row == 1 && (s_k & 7) == 0 && al) return ST_KCOL;
-    return ST_SCALAR;
-}
-
-// One K chunk of a ROWS x TC_BK operand tile: the loads into registers (NV
-// 16-byte vectors a thread, all issued before any is used, so their
-// latencies overlap one another and the previous chunk's products) ...
-template <int ROWS>
-struct TcStage {
-    static constexpr int NV = ROWS * (TC_BK / 8) / 128;
-    uint4 v[NV];
-
-    __device__ __forceinline__ void load(int mode, const __nv_bfloat16* __restrict__ src, long s_row, long s_k,
-                                         int r0, int R, int k0, int K) {
-        const __nv_bfloat16 z = __float2bfloat16(0.f);
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int e = threadIdx.x + 128 * i;
-            v[i] = make_uint4(0u, 0u, 0u, 0u);
-            __nv_bfloat16* t = reinterpret_cast<__nv_bfloat16*>(&v[i]);
-            if (mode == ST_KROW) {  // row r, k-octet kc
-                const int r = e / TC_KO, gr = r0 + r, gk = k0 + 8 * (e % TC_KO);
-                if (gr < R && gk + 8 <= K)
-                    v[i] = *reinterpret_cast<const uint4*>(src + (long)gr * s_row + gk);
-                else if (gr < R)
-                    for (int j = 0; j < 8; ++j) t[j] = gk + j < K ? src[(long)gr * s_row + gk + j] : z;
-            } else if (mode == ST_KCOL) {  // rows 8 g .. 8 g + 7 at one k
-                const int g = e / TC_BK, gr = r0 + 8 * g, gk = k0 + (e - g * TC_BK);
-                if (gk < K && gr + 8 <= R)
-                    v[i] = *reinterpret_cast<const uint4*>(src + (long)gk * s_k + gr);
-                else if (gk < K)
-                    for (int j = 0; j < 8; ++j) t[j] = gr + j < R ? src[(long)gk * s_k + gr + j] : z;
-            }
-        }
-    }
-
-    // ... then the stores into the K-major core-matrix layout (the element
-    // by element mode loads and stores here)
-    __device__ __forceinline__ void store(int mode, __nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src,
-                                          long s_row, long s_k, int r0, int R, int k0, int K) const {
-        if (mode == ST_SCALAR) {
-            const __nv_bfloat16 z = __float2bfloat16(0.f);
-            for (int e = threadIdx.x; e < ROWS * TC_BK; e += 128) {
-                const int r = e / TC_BK, k = e - r * TC_BK;
-                const int gr = r0 + r, gk = k0 + k;
-                dst[tc_at(r, k)] = (gr < R && gk < K) ? src[(long)gr * s_row + (long)gk * s_k] : z;
-            }
-            return;
-        }
-#pragma unroll
-        for (int i = 0; i < NV; ++i) {
-            const int e = threadIdx.x + 128 * i;
-            if (mode == ST_KROW) {
-                *reinterpret_cast<uint4*>(dst + tc_at(e / TC_KO, 8 * (e % TC_KO))) = v[i];
-            } else {
-                const int g = e / TC_BK, k = e - g * TC_BK;
-                const __nv_bfloat16* t = reinterpret_cast<const __nv_bfloat16*>(&v[i]);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) dst[tc_at(8 * g + j, k)] = t[j];
-            }
-        }
-    }
+struct Gemm {
+    const __nv_bfloat16* A = nullptr;
+    long sam = 0, sak = 0;
+    const float* Af = nullptr;  // FP32 rows of K in place of A
+    const __nv_bfloat16* B = nullptr;
+    long sbk = 0, sbn = 0;
+    int M = 0, N = 0, K = 0, epi = EPI_PLAIN;
+    float* C = nullptr;  // EPI_PLAIN: the product [M x N]
+    // EPI_HIDDEN: z = product + bias into Z (nullable), silu(z) into H.
+    // EPI_OUT: product + bias into Y; with T, 2 (y - T) / (M N) into D and H
+    // (row r of the batch is row tidx[r] of T, or r).
+    // EPI_BACK: product times silu'(Z) into D and H
+    const float* bias = nullptr;
+    float* Z = nullptr;
+    __nv_bfloat16* H = nullptr;
+    float* Y = nullptr;
+    const float* T = nullptr;
+    const int* tidx = nullptr;
+    float* D = nullptr;
+    int tm = 0, tiles = 0;  // tiles along M, in all
 };
-
-template <int BN>
-__global__ void __launch_bounds__(128) k_gemm_tc(const __nv_bfloat16* __restrict__ A, long sam, long sak,
-                                                 const __nv_bfloat16* __restrict__ B, long sbk, long sbn,
-                                                 float* __restrict__ C, int ldc, int M, int N, int K) {
-    using namespace mirage::tc05;
-    constexpr int TCOLS = BN < 32 ? 32 : BN;  // a power of two >= 32
-    constexpr uint32_t ID = idesc(FMT_BF16, TC_BM, BN);
-    extern __shared__ __align__(128) unsigned char tc_sm[];
-    __nv_bfloat16* sA = reinterpret_cast<__nv_bfloat16*>(tc_sm);
-    __nv_bfloat16* sB = sA + TC_BM * TC_BK;
-    uint64_t* bar = reinterpret_cast<uint64_t*>(sB + BN * TC_BK);
-    uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 1);
-    const int m0 = blockIdx.x * TC_BM, n0 = blockIdx.y * BN;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // B(k, n) is staged as rows n: row stride sbn, k stride sbk
-    const int ma = stage_mode(A, sam, sak), mb = stage_mode(B, sbn, sbk);
-    TcStage<TC_BM> ra;
-    TcStage<BN> rb;
-    ra.load(ma, A, sam, sak, m0, M, 0, K);
-    rb.load(mb, B, sbn, sbk, n0, N, 0, K);
-    if (warp == 0) tmem_alloc(slot, TCOLS);
-    if (threadIdx.x == 0) bar_init(bar, 1);
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    const uint32_t tmem = *slot;
-    bool ok = true;
-    uint32_t phase = 0;
-    for (int k0 = 0; k0 < K && ok; k0 += TC_BK) {
-        ra.store(ma, sA, A, sam, sak, m0, M, k0, K);
-        rb.store(mb, sB, B, sbn, sbk, n0, N, k0, K);
-        fence_async_smem();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            fence_after_sync();
-#pragma unroll
-            for (int s = 0; s < TC_BK / 16; ++s) {
-                // K step s: core-matrix columns 2s and 2s + 1 (128 B apart),
-                // 8-row groups TC_KO * 128 B apart
-                const uint64_t da = sdesc(saddr(sA) + s * 256, 128, TC_KO * 128);
-                const uint64_t db = sdesc(saddr(sB) + s * 256, 128, TC_KO * 128);
-                mma_bf16(tmem, da, db, ID, (k0 > 0 || s > 0) ? 1u : 0u);
-            }
-            commit(bar);
-        }
-        if (k0 + TC_BK < K) {  // the next chunk's loads overlap these products
-            ra.load(ma, A, sam, sak, m0, M, k0 + TC_BK, K);
-            rb.load(mb, B, sbn, sbk, n0, N, k0 + TC_BK, K);
-        }
-        ok = __syncthreads_and(bar_wait(bar, phase)) != 0;  // one decision for the whole CTA
-        phase ^= 1;
-        fence_after_sync();
-    }
-    if (!ok) bar_wait(bar, phase ^ 1);  // (bounded) for the MMAs still in flight
-    const int row = m0 + warp * 32 + lane;
-#pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 16) {
-        float v[16];
-        ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-        if (row < M) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const int col = n0 + c0 + j;
-                if (col < N) C[(long)row * ldc + col] = (ok && K > 0) ? v[j] : (K > 0 ? __int_as_float(0x7fc00000) : 0.f);
-            }
-        }
-    }
-    fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tmem_free(tmem, TCOLS);
-}
+struct LayerArgs {
+    Gemm g[2];
+    // column sums of S [srows x scols] into sum (fixed order), 32 columns a CTA
+    const float* S = nullptr;
+    int srows = 0, scols = 0;
+    float* sum = nullptr;
+    long long* inc = nullptr;  // incremented by one
+};
 
 __device__ __forceinline__ float silu_f(float z) { return z / (1.f + __expf(-z)); }
 __device__ __forceinline__ float silu_g(float z) {
@@ -203,26 +99,237 @@ __device__ __forceinline__ float silu_g(float z) {
     return s * (1.f + z * (1.f - s));
 }
 
-// x (FP32) -> BF16 activations; with idx, row j of the batch is row idx[j] of x
-__global__ void k_to_bf16(const float* __restrict__ x, const int* __restrict__ idx, int cols,
-                          __nv_bfloat16* __restrict__ a, long n) {
-    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const long src = idx ? (long)idx[i / cols] * cols + i % cols : i;
-    a[i] = __float2bfloat16(x[src]);
+// Launches of a chain are programmatic dependents of each other: a kernel lets
+// the next one start (its CTAs become resident, allocate and wait) as soon as
+// all its own run, and waits itself for the previous one's results before it
+// reads or writes anything that they share
+__device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// 8 x 8 transpose of BF16: v[i] holds row i (8 values); row j of the result
+__device__ __forceinline__ uint4 tc_column(const uint4 (&v)[8], int j) {
+    const unsigned sel = (j & 1) ? 0x7632u : 0x5410u;
+    auto word = [&](const uint4& a) { return (j >> 1) == 0 ? a.x : (j >> 1) == 1 ? a.y : (j >> 1) == 2 ? a.z : a.w; };
+    return make_uint4(__byte_perm(word(v[0]), word(v[1]), sel), __byte_perm(word(v[2]), word(v[3]), sel),
+                      __byte_perm(word(v[4]), word(v[5]), sel), __byte_perm(word(v[6]), word(v[7]), sel));
 }
 
-// Z += b (per column); hidden layers: A = bf16(silu(Z)); output layer: Y = Z
-__global__ void k_bias_act(float* __restrict__ Z, const float* __restrict__ b, int n, int cols, int hidden,
-                           __nv_bfloat16* __restrict__ Aout, float* __restrict__ Y) {
+// ROWS rows x kn (a multiple of 16, at most TC_BK) of an operand view into the
+// core matrices at dst; zeros beyond K (rows beyond R only reach outputs that
+// are not stored, and are left as they are)
+template <int ROWS>
+__device__ __forceinline__ void tc_stage(unsigned char* dst, const __nv_bfloat16* __restrict__ src, long s_row, long s_k,
+                                         const float* __restrict__ srcf, int r0, int R, int k0, int K, int kn) {
+    const bool al = ((uintptr_t)src & 15) == 0;
+    const int tid = threadIdx.x, ko = kn >> 3;
+    if (!srcf && s_k == 1 && (s_row & 7) == 0 && al && k0 + kn <= K) {
+        // rows contiguous along k: copied straight to shared memory, eight lanes
+        // taking 128 consecutive bytes of a row
+        const int rows = min(ROWS, R - r0);
+        const __nv_bfloat16* s0 = src + (long)r0 * s_row + k0;
+#pragma unroll
+        for (int i = 0; i < ROWS * (TC_BK / 8) / TC_T; ++i) {
+            const int e = tid + TC_T * i, o = e % (TC_BK / 8), r = e / (TC_BK / 8);
+            if (o < ko && r < rows)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(mirage::tc05::saddr(dst + tc_row(r, o))),
+                             "l"(s0 + (long)r * s_row + 8 * o)
+                             : "memory");
+        }
+        return;
+    }
+    if (!srcf && s_row == 1 && (s_k & 7) == 0 && al && (r0 + ROWS <= R || ((R - r0) & 7) == 0) && k0 + kn <= K) {
+        // rows contiguous at one k: 8 x 8 blocks, turned in registers
+        constexpr int MB = ROWS / 8, MQ = MB < 8 ? MB : 8;  // 8 row blocks x 4 k-octets a warp
+#pragma unroll 1
+        for (int e = tid; e < MB * ((ko + 3) & ~3); e += TC_T) {
+            const int q = e / (4 * MQ), mb = e % MQ + MQ * (q % (MB / MQ)), kb = e / MQ % 4 + 4 * (q / (MB / MQ));
+            if (kb >= ko || r0 + 8 * mb >= R) continue;
+            uint4 v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                v[i] = *reinterpret_cast<const uint4*>(src + (long)(k0 + 8 * kb + i) * s_k + r0 + 8 * mb);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) *reinterpret_cast<uint4*>(dst + tc_row(8 * mb + j, kb)) = tc_column(v, j);
+        }
+        return;
+    }
+    // any other view, element by element
+    const __nv_bfloat16 z = __float2bfloat16(0.f);
+    const int rows = min(ROWS, R - r0);
+    for (int e = tid; e < rows * kn; e += TC_T) {
+        const int r = e / kn, k = e - r * kn, gr = r0 + r, gk = k0 + k;
+        __nv_bfloat16 x = z;
+        if (gk < K)
+            x = srcf ? __float2bfloat16(srcf[(long)gr * K + gk]) : src[(long)gr * s_row + (long)gk * s_k];
+        *reinterpret_cast<__nv_bfloat16*>(dst + tc_row(r, k >> 3) + (k & 7) * 2) = x;
+    }
+}
+
+template <int BN>
+__device__ void tc_tile(const Gemm& q, int tile, unsigned char* sm) {
+    using namespace mirage::tc05;
+    constexpr int TCOLS = BN < 32 ? 32 : BN;  // a power of two >= 32
+    constexpr uint32_t ID = idesc(FMT_BF16, TC_BM, BN);
+    unsigned char* sA = sm;
+    unsigned char* sB = sA + TC_BM / 8 * TC_SBO;
+    uint64_t* bar = reinterpret_cast<uint64_t*>(sB + BN / 8 * TC_SBO);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(bar + 1);
+    const int m0 = (tile % q.tm) * TC_BM, n0 = (tile / q.tm) * BN;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    static_assert(TC_BM * (BN + 1) * 4 <= TC_BM / 8 * TC_SBO, "the accumulator tile fits where A was staged");
+    if (warp == 0) tmem_alloc(slot, TCOLS);
+    if (threadIdx.x == 32) bar_init(bar, 1);
+    dep_wait();
+    bool ok = true;
+    uint32_t phase = 0, tmem = 0;
+    for (int k0 = 0; k0 < q.K && ok; k0 += TC_BK) {
+        const int kn = min(TC_BK, (q.K - k0 + 15) & ~15);
+        tc_stage<TC_BM>(sA, q.A, q.sam, q.sak, q.Af, m0, q.M, k0, q.K, kn);
+        tc_stage<BN>(sB, q.B, q.sbn, q.sbk, nullptr, n0, q.N, k0, q.K, kn);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        fence_async_smem();
+        fence_before_sync();
+        __syncthreads();
+        fence_after_sync();
+        tmem = *slot;
+        if (threadIdx.x == 0) {
+            for (int s = 0; s < kn / 16; ++s) {
+                const uint64_t da = sdesc(saddr(sA) + s * 2 * TC_LBO, TC_LBO, TC_SBO);
+                const uint64_t db = sdesc(saddr(sB) + s * 2 * TC_LBO, TC_LBO, TC_SBO);
+                mma_bf16(tmem, da, db, ID, (k0 > 0 || s > 0) ? 1u : 0u);
+            }
+            commit(bar);
+        }
+        ok = __syncthreads_and(bar_wait(bar, phase)) != 0;  // one decision for the whole CTA
+        phase ^= 1;
+        fence_after_sync();
+    }
+    if (!ok) bar_wait(bar, phase ^ 1);  // (bounded) for the MMAs still in flight
+    // accumulator to shared memory (warps w and w + 4 share tensor-memory lanes
+    // 32 (w mod 4) .. and take the columns in turns of 16), then the epilogue
+    // along rows: a thread's global accesses are its neighbours'
+    constexpr int LD = BN + 1;
+    float* tile_sm = reinterpret_cast<float*>(sm);
+    __syncthreads();  // (the products have read the operands)
+#pragma unroll 1
+    for (int c0 = 16 * (warp >> 2); c0 < BN; c0 += 32) {
+        float v[16];
+        ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0, v);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) tile_sm[((warp & 3) * 32 + lane) * LD + c0 + j] = v[j];
+    }
+    __syncthreads();
+    const float nan = __int_as_float(0x7fc00000);
+    const int rows = min(TC_BM, q.M - m0), cl = threadIdx.x % BN, rl = threadIdx.x / BN, col = n0 + cl;
+    if (col < q.N) {
+        const long i0 = (long)(m0 + rl) * q.N + col, step = (long)(TC_T / BN) * q.N;
+        const float* ts = tile_sm + rl * LD + cl;
+        // f(i, product) of this thread's elements, eight at a time
+        auto each = [&](auto&& f) {
+            constexpr int NR = TC_BM * BN / TC_T, U = NR < 8 ? NR : 8;
+#pragma unroll 1
+            for (int j0 = 0; j0 < NR; j0 += U)
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int j = j0 + u;
+                    if (rl + j * (TC_T / BN) < rows) f(i0 + j * step, ok ? ts[j * (TC_T / BN) * LD] : nan, m0 + rl + j * (TC_T / BN));
+                }
+        };
+        const float bias = q.bias ? q.bias[col] : 0.f;
+        if (q.epi == EPI_PLAIN) {
+            float* C = q.C;
+            each([&](long i, float p, int) { C[i] = p; });
+        } else if (q.epi == EPI_HIDDEN) {
+            float* Z = q.Z;
+            __nv_bfloat16* H = q.H;
+            each([&](long i, float p, int) {
+                const float z = p + bias;
+                if (Z) Z[i] = z;
+                H[i] = __float2bfloat16(silu_f(z));
+            });
+        } else if (q.epi == EPI_OUT) {
+            each([&](long i, float p, int r) {
+                const float y = p + bias;
+                q.Y[i] = y;
+                if (q.T) {
+                    const float d = y - q.T[(long)(q.tidx ? q.tidx[r] : r) * q.N + col];
+                    const float g = 2.f * d / (float)((long)q.M * q.N);
+                    q.D[i] = g;
+                    q.H[i] = __float2bfloat16(g);
+                }
+            });
+        } else {
+            const float* __restrict__ Z = q.Z;
+            float* __restrict__ D = q.D;
+            __nv_bfloat16* __restrict__ H = q.H;
+            each([&](long i, float p, int) {
+                const float d = p * silu_g(Z[i]);
+                D[i] = d;
+                H[i] = __float2bfloat16(d);
+            });
+        }
+    }
+    fence_before_sync();
+    __syncthreads();
+    if (warp == 0) {
+        fence_after_sync();
+        tmem_free(tmem, TCOLS);
+    }
+}
+
+// sum[j] = sum_m S[m][j] for 32 columns, added in the order of m: the rows
+// arrive in shared memory 256 at a time, one thread adds each column
+__device__ void col_sums(const float* __restrict__ S, int rows, int cols, int j0, float* __restrict__ sum, float* sm) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    dep_wait();
+    float s = 0.f;
+    for (int m0 = 0; m0 < rows; m0 += 256) {
+        float v[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const int m = m0 + warp * 32 + i;
+            v[i] = m < rows && j0 + lane < cols ? S[(long)m * cols + j0 + lane] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) sm[(warp * 32 + i) * 32 + lane] = v[i];
+        __syncthreads();
+        if (warp == 0) {
+            const int n = min(256, rows - m0);
+#pragma unroll 16
+            for (int i = 0; i < n; ++i) s += sm[i * 32 + lane];
+        }
+        __syncthreads();
+    }
+    if (warp == 0 && j0 + lane < cols) sum[j0 + lane] = s;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(TC_T) k_layer(const __grid_constant__ LayerArgs a) {
+    extern __shared__ __align__(128) unsigned char tc_sm[];
+    dep_launch();
+    int b = blockIdx.x;
+    if (b == 0 && threadIdx.x == 0 && a.inc) {
+        dep_wait();
+        *a.inc += 1;
+    }
+    if (b < a.g[0].tiles) {
+        tc_tile<BN>(a.g[0], b, tc_sm);
+        return;
+    }
+    b -= a.g[0].tiles;
+    if (b < a.g[1].tiles) {
+        tc_tile<BN>(a.g[1], b, tc_sm);
+        return;
+    }
+    col_sums(a.S, a.srows, a.scols, 32 * (b - a.g[1].tiles), a.sum, reinterpret_cast<float*>(tc_sm));
+}
+
+// x (FP32) -> BF16 activations
+__global__ void k_to_bf16(const float* __restrict__ x, __nv_bfloat16* __restrict__ a, long n) {
+    dep_launch();
+    dep_wait();
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= (long)n * cols) return;
-    const float z = Z[i] + b[i % cols];
-    Z[i] = z;
-    if (hidden)
-        Aout[i] = __float2bfloat16(silu_f(z));
-    else
-        Y[i] = z;
+    if (i < n) a[i] = __float2bfloat16(x[i]);
 }
 
 // dY = 2 (Y - T) / (n cols); loss partial sums.  With idx, row j of the
@@ -230,6 +337,8 @@ __global__ void k_bias_act(float* __restrict__ Z, const float* __restrict__ b, i
 __global__ void k_loss_grad(const float* __restrict__ Y, const float* __restrict__ T, const int* __restrict__ idx,
                             int cols, long total, float* __restrict__ dZ, __nv_bfloat16* __restrict__ dZh,
                             double* __restrict__ loss) {
+    dep_launch();
+    dep_wait();
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     double l = 0.0;
     if (i < total) {
@@ -245,51 +354,14 @@ __global__ void k_loss_grad(const float* __restrict__ Y, const float* __restrict
     }
 }
 
-// dZ = dA * silu'(Z) (hidden layer), also its BF16 copy
-__global__ void k_act_back(const float* __restrict__ dA, const float* __restrict__ Z, long total,
-                           float* __restrict__ dZ, __nv_bfloat16* __restrict__ dZh) {
-    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= total) return;
-    const float d = dA[i] * silu_g(Z[i]);
-    dZ[i] = d;
-    dZh[i] = __float2bfloat16(d);
-}
-
-// db[j] = sum_m dZ[m][j] (fixed order, one thread per column)
-__global__ void k_colsum(const float* __restrict__ dZ, int n, int cols, float* __restrict__ db) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= cols) return;
-    float s = 0.f;
-    for (int m = 0; m < n; ++m) s += dZ[(long)m * cols + j];
-    db[j] = s;
-}
-
 // Adam on every parameter; refresh the BF16 copy of the weights
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, long n, float lr, float b1, float b2, float eps, float c1, float c2,
                        __nv_bfloat16* __restrict__ ph, const unsigned char* __restrict__ is_w) {
+    dep_launch();
+    dep_wait();
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float w = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    p[i] = w;
-    if (is_w[i]) ph[i] = __float2bfloat16(w);
-}
-
-// Adam whose bias corrections follow the device step counter (steps taken
-// so far, before this one), for the device-side training loop
-__global__ void k_adam_dev(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                           float* __restrict__ v, long n, float lr, float b1, float b2, float eps,
-                           const long long* __restrict__ dstep, __nv_bfloat16* __restrict__ ph,
-                           const unsigned char* __restrict__ is_w) {
-    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float s = (float)(*dstep + 1);
-    const float c1 = 1.f - powf(b1, s), c2 = 1.f - powf(b2, s);
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
@@ -308,15 +380,52 @@ __device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
 }
-__global__ void k_sample_rows(int* __restrict__ idx, int batch, int n, unsigned long long seed,
-                              const long long* __restrict__ dstep) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= batch) return;
-    const unsigned long long key =
-        seed * 0x9E3779B97F4A7C15ull + ((unsigned long long)*dstep << 24) + (unsigned long long)j;
-    idx[j] = (int)(mix64(key) % (unsigned long long)n);
+struct Draw {
+    int* idx;                // the rows' numbers ...
+    __nv_bfloat16* a;        // ... and the rows (BF16)
+    const float* x;
+    int batch, n, cols;
+    unsigned long long seed;
+};
+__device__ __forceinline__ void draw_rows(const Draw& d, long long step, long i) {
+    if (i >= (long)d.batch * d.cols) return;
+    const int j = (int)(i / d.cols), c = (int)(i - (long)j * d.cols);
+    const unsigned long long key = d.seed * 0x9E3779B97F4A7C15ull + ((unsigned long long)step << 24) + (unsigned long long)j;
+    const int row = (int)(mix64(key) % (unsigned long long)d.n);
+    if (c == 0) d.idx[j] = row;
+    d.a[i] = __float2bfloat16(d.x[(long)row * d.cols + c]);
 }
-__global__ void k_step_inc(long long* dstep) { *dstep += 1; }
+// the rows of the first step of a training call
+__global__ void k_draw(Draw d, const long long* __restrict__ dstep) {
+    draw_rows(d, *dstep, blockIdx.x * (long)blockDim.x + threadIdx.x);
+}
+
+// The end of a step of the device-side training loop: Adam with the bias
+// corrections of the device step counter (this step included), and, on the
+// CTAs after the parameters' `nb`, the next step's rows
+__global__ void k_adam_dev(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
+                           float* __restrict__ v, long n, float lr, float b1, float b2, float eps,
+                           const long long* __restrict__ dstep, __nv_bfloat16* __restrict__ ph,
+                           const unsigned char* __restrict__ is_w, unsigned nb, Draw d) {
+    dep_launch();
+    dep_wait();
+    if (blockIdx.x >= nb) {
+        draw_rows(d, *dstep, (blockIdx.x - nb) * (long)blockDim.x + threadIdx.x);
+        return;
+    }
+    const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float s = (float)*dstep;
+    const float c1 = 1.f - powf(b1, s), c2 = 1.f - powf(b2, s);
+    const float gi = g[i];
+    const float mi = b1 * m[i] + (1.f - b1) * gi;
+    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    const float w = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = w;
+    if (is_w[i]) ph[i] = __float2bfloat16(w);
+}
 
 __global__ void k_params_bf16(const float* __restrict__ p, __nv_bfloat16* __restrict__ ph, long n) {
     const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
@@ -355,14 +464,22 @@ struct mirage_mlp {
     int step = 0;
     float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     Buf P, PH, M, V, G, ISW;   // params FP32, BF16 copy, Adam m, v, grads, weight mask
-    Buf Z, A, DZ, DZH, DA, LOSS;  // per-batch work (grown on demand)
+    Buf Z, A, DZ, DZH, DA, LOSS;  // per-batch work (grown on demand; DZ and DZH twice: a layer's and the next one's)
     Buf IDX, DSTEP;            // device-side training loop: minibatch rows, step counter
     cudaStream_t cap = nullptr;  // private stream on which the training step is captured
     long cap_rows = 0;
+    int maxw = 0;              // widest layer
     std::vector<long> z_off, a_off;  // per layer offsets into Z / A (elements)
 };
 
 namespace {
+
+// dynamic shared memory of a layer launch: a product's tile or the column
+// sums' rows
+template <int BN>
+constexpr int layer_smem() {
+    return tc_smem_bytes<BN>() > 256 * 32 * 4 ? tc_smem_bytes<BN>() : 256 * 32 * 4;
+}
 
 int ensure_batch(mirage_mlp* m, int n) {
     if (n <= m->cap_rows) return MIRAGE_OK;
@@ -372,7 +489,7 @@ int ensure_batch(mirage_mlp* m, int n) {
     int maxw = 0;
     for (int l = 0; l <= m->L; ++l) {
         m->a_off[l] = at;
-        at += (long)n * m->dims[l];
+        at += ((long)n * m->dims[l] + 7) & ~7L;  // (16-byte rows stay aligned)
         maxw = std::max(maxw, m->dims[l]);
         if (l > 0) {
             m->z_off[l] = zt;
@@ -382,97 +499,167 @@ int ensure_batch(mirage_mlp* m, int n) {
     int r;
     if ((r = m->Z.ensure(sizeof(float) * zt))) return r;
     if ((r = m->A.ensure(sizeof(__nv_bfloat16) * at))) return r;
-    if ((r = m->DZ.ensure(sizeof(float) * (long)n * maxw))) return r;
-    if ((r = m->DZH.ensure(sizeof(__nv_bfloat16) * (long)n * maxw))) return r;
+    if ((r = m->DZ.ensure(2 * sizeof(float) * (((long)n * maxw + 7) & ~7L)))) return r;
+    if ((r = m->DZH.ensure(2 * sizeof(__nv_bfloat16) * (((long)n * maxw + 7) & ~7L)))) return r;
     if ((r = m->DA.ensure(sizeof(float) * (long)n * maxw))) return r;
     if ((r = m->LOSS.ensure(sizeof(double)))) return r;
+    m->maxw = maxw;
     m->cap_rows = n;
     return MIRAGE_OK;
 }
 
-template <int BN>
-int gemm_tc(const __nv_bfloat16* A, long sam, long sak, const __nv_bfloat16* B, long sbk, long sbn, float* C, int ldc,
-            int M, int N, int K, cudaStream_t st) {
-    constexpr int smem = tc_smem_bytes<BN>();
-    const dim3 grid((unsigned)((M + TC_BM - 1) / TC_BM), (unsigned)((N + BN - 1) / BN));
-    k_gemm_tc<BN><<<grid, 128, smem, st>>>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K);
-    MCK(cudaGetLastError());
-    return MIRAGE_OK;
-}
-
-// raises the product kernels' shared-memory limit on the current device
-// (once per network, outside any stream capture)
+// raises the layer kernels' shared-memory limit on the current device (once
+// per network, outside any stream capture)
 int gemm_setup() {
-    MCK(cudaFuncSetAttribute(k_gemm_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_bytes<16>()));
-    MCK(cudaFuncSetAttribute(k_gemm_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_bytes<32>()));
-    MCK(cudaFuncSetAttribute(k_gemm_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc_smem_bytes<64>()));
+    MCK(cudaFuncSetAttribute(k_layer<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_smem<16>()));
+    MCK(cudaFuncSetAttribute(k_layer<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, layer_smem<32>()));
     return MIRAGE_OK;
 }
 
-// the N tile: 16 or 32 for the narrow output layer, else 64 columns (the
-// 256-wide layers run in four tiles: more CTAs, each with a shorter
-// staging pass)
-int gemm(const __nv_bfloat16* A, long sam, long sak, const __nv_bfloat16* B, long sbk, long sbn, float* C, int ldc,
-         int M, int N, int K, cudaStream_t st) {
-    if (M <= 0 || N <= 0) return MIRAGE_OK;
-    if (N <= 16) return gemm_tc<16>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, st);
-    if (N <= 32) return gemm_tc<32>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, st);
-    return gemm_tc<64>(A, sam, sak, B, sbk, sbn, C, ldc, M, N, K, st);
+// launch as a programmatic dependent of the stream's previous launch
+template <class... P, class... Q>
+cudaError_t launch_dep(void (*fn)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, Q... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, P(args)...);
 }
 
-// forward pass storing Z (FP32) and A (BF16); Y (FP32) written to y.  With
-// idx, batch row j is row idx[j] of x.
-int forward_pass(mirage_mlp* m, const float* x, int n, float* y, cudaStream_t st, const int* idx = nullptr) {
+// one launch of a layer's work, in N tiles of 16 columns for narrow products
+// and 32 for the others (the 256-wide layers run in eight: more CTAs, each with
+// a shorter epilogue)
+template <int BN>
+int launch_layer_bn(LayerArgs& a, cudaStream_t st) {
+    unsigned grid = 0;
+    for (Gemm& g : a.g) {
+        g.tm = (g.M + TC_BM - 1) / TC_BM;
+        g.tiles = g.M > 0 && g.N > 0 ? g.tm * ((g.N + BN - 1) / BN) : 0;
+        grid += (unsigned)g.tiles;
+    }
+    if (a.S) grid += (unsigned)((a.scols + 31) / 32);
+    if (!grid) return MIRAGE_OK;
+    MCK(launch_dep(k_layer<BN>, grid, TC_T, layer_smem<BN>(), st, a));
+    return MIRAGE_OK;
+}
+int launch_layer(LayerArgs& a, cudaStream_t st) {
+    const int N = a.g[0].N;  // (the second product has the same width)
+    if (N <= 16) return launch_layer_bn<16>(a, st);
+    return launch_layer_bn<32>(a, st);
+}
+
+// The forward pass, one launch a layer: z_l (FP32, kept for a backward pass)
+// and a_l (BF16) of the hidden layers, y of the last.  With idx, batch row j
+// is row idx[j] of x; with tgt the last layer also leaves the loss gradient in
+// DZ and DZH; inc is incremented (device step counter).
+int forward_pass(mirage_mlp* m, const float* x, int n, float* y, cudaStream_t st, bool keep = false, const int* idx = nullptr,
+                 const float* tgt = nullptr, long long* inc = nullptr) {
     int r;
     if ((r = ensure_batch(m, n))) return r;
     float* Z = (float*)m->Z.p;
     __nv_bfloat16* A = (__nv_bfloat16*)m->A.p;
     const float* P = (const float*)m->P.p;
     const __nv_bfloat16* PH = (const __nv_bfloat16*)m->PH.p;
-    k_to_bf16<<<blocks((long)n * m->dims[0], 256), 256, 0, st>>>(x, idx, m->dims[0], A, (long)n * m->dims[0]);
+    if (keep && !idx) {  // the backward pass reads the input as BF16 too (drawn rows already are)
+        MCK(launch_dep(k_to_bf16, blocks((long)n * m->dims[0], 256), 256, 0, st, x, A, (long)n * m->dims[0]));
+    }
     for (int l = 1; l <= m->L; ++l) {
         const int in = m->dims[l - 1], out = m->dims[l];
+        LayerArgs a;
+        Gemm& g = a.g[0];
         // Z_l = A_{l-1} W_l^T : A(m, k) = A[m in + k], B(k, j) = W[j in + k]
-        if ((r = gemm(A + m->a_off[l - 1], in, 1, PH + m->w_off[l - 1], 1, in, Z + m->z_off[l], out, n, out, in, st)))
-            return r;
-        const bool hidden = l < m->L;
-        k_bias_act<<<blocks((long)n * out, 256), 256, 0, st>>>(Z + m->z_off[l], P + m->b_off[l - 1], n, out, hidden,
-                                                               A + m->a_off[l], y);
-        MCK(cudaGetLastError());
+        if (l == 1 && !keep) g.Af = x;
+        g.A = A + m->a_off[l - 1];
+        g.sam = in;
+        g.sak = 1;
+        g.B = PH + m->w_off[l - 1];
+        g.sbk = 1;
+        g.sbn = in;
+        g.M = n;
+        g.N = out;
+        g.K = in;
+        g.bias = P + m->b_off[l - 1];
+        if (l < m->L) {
+            g.epi = EPI_HIDDEN;
+            g.Z = keep ? Z + m->z_off[l] : nullptr;
+            g.H = A + m->a_off[l];
+        } else {
+            g.epi = EPI_OUT;
+            g.Y = y;
+            g.T = tgt;
+            g.tidx = idx;
+            g.D = (float*)m->DZ.p;
+            g.H = (__nv_bfloat16*)m->DZH.p;
+        }
+        if (l == 1) a.inc = inc;
+        if ((r = launch_layer(a, st))) return r;
     }
     return MIRAGE_OK;
 }
 
 // gradients of the MSE into m->G (and the loss into m->LOSS if wanted)
 int backward_pass(mirage_mlp* m, const float* x, const float* tgt, int n, float* yscratch, bool want_loss,
-                  cudaStream_t st, const int* idx = nullptr) {
+                  cudaStream_t st, const int* idx = nullptr, long long* inc = nullptr) {
     int r;
-    if ((r = forward_pass(m, x, n, yscratch, st, idx))) return r;
+    if ((r = forward_pass(m, x, n, yscratch, st, true, idx, want_loss ? nullptr : tgt, inc))) return r;
     float* Z = (float*)m->Z.p;
     __nv_bfloat16* A = (__nv_bfloat16*)m->A.p;
-    float* DZ = (float*)m->DZ.p;
-    __nv_bfloat16* DZH = (__nv_bfloat16*)m->DZH.p;
-    float* DA = (float*)m->DA.p;
     float* G = (float*)m->G.p;
     const __nv_bfloat16* PH = (const __nv_bfloat16*)m->PH.p;
-    double* loss = want_loss ? (double*)m->LOSS.p : nullptr;
-    if (loss) MCK(cudaMemsetAsync(loss, 0, sizeof(double), st));
     const int outL = m->dims[m->L];
-    k_loss_grad<<<blocks((long)n * outL, 256), 256, 0, st>>>(yscratch, tgt, idx, outL, (long)n * outL, DZ, DZH,
-                                                             loss);
-    MCK(cudaGetLastError());
-    for (int l = m->L; l >= 1; --l) {
+    if (want_loss) {
+        double* loss = (double*)m->LOSS.p;
+        MCK(cudaMemsetAsync(loss, 0, sizeof(double), st));
+        MCK(launch_dep(k_loss_grad, blocks((long)n * outL, 256), 256, 0, st, yscratch, tgt, idx, outL, (long)n * outL,
+                       (float*)m->DZ.p, (__nv_bfloat16*)m->DZH.p, loss));
+    }
+    const long half = ((long)m->cap_rows * m->maxw + 7) & ~7L;  // a layer's part of DZ and DZH
+    for (int l = m->L, cur = 0; l >= 1; --l, cur ^= 1) {
         const int in = m->dims[l - 1], out = m->dims[l];
+        float *dz = (float*)m->DZ.p + cur * half, *dzn = (float*)m->DZ.p + (cur ^ 1) * half;
+        __nv_bfloat16 *dzh = (__nv_bfloat16*)m->DZH.p + cur * half, *dzhn = (__nv_bfloat16*)m->DZH.p + (cur ^ 1) * half;
+        LayerArgs a;
         // dW_l = dZ^T A_{l-1}: [out x in];  A(mm, k) = dZ[k out + mm], B(k, j) = A_{l-1}[k in + j]
-        if ((r = gemm(DZH, 1, out, A + m->a_off[l - 1], in, 1, G + m->w_off[l - 1], in, out, in, n, st))) return r;
-        k_colsum<<<blocks(out, 128), 128, 0, st>>>(DZ, n, out, G + m->b_off[l - 1]);
-        MCK(cudaGetLastError());
+        Gemm& w = a.g[0];
+        w.A = dzh;
+        w.sam = 1;
+        w.sak = out;
+        w.B = A + m->a_off[l - 1];
+        w.sbk = in;
+        w.sbn = 1;
+        w.C = G + m->w_off[l - 1];
+        w.M = out;
+        w.N = in;
+        w.K = n;
+        // db_l: column sums of dZ
+        a.S = dz;
+        a.srows = n;
+        a.scols = out;
+        a.sum = G + m->b_off[l - 1];
         if (l > 1) {
             // dA_{l-1} = dZ W_l: A(mm, k) = dZ[mm out + k], B(k, j) = W[k in + j]
-            if ((r = gemm(DZH, out, 1, PH + m->w_off[l - 1], in, 1, DA, in, n, in, out, st))) return r;
-            k_act_back<<<blocks((long)n * in, 256), 256, 0, st>>>(DA, Z + m->z_off[l - 1], (long)n * in, DZ, DZH);
-            MCK(cudaGetLastError());
+            Gemm& d = a.g[1];
+            d.A = dzh;
+            d.sam = out;
+            d.sak = 1;
+            d.B = PH + m->w_off[l - 1];
+            d.sbk = in;
+            d.sbn = 1;
+            d.M = n;
+            d.N = in;
+            d.K = out;
+            d.epi = EPI_BACK;
+            d.Z = Z + m->z_off[l - 1];
+            d.D = dzn;
+            d.H = dzhn;
         }
+        if ((r = launch_layer(a, st))) return r;
     }
     return MIRAGE_OK;
 }
@@ -598,10 +785,9 @@ int mirage_mlp_train_step(mirage_mlp_t* m, const float* x, const float* t, int n
     if (r) return r;
     m->step += 1;
     const float c1 = 1.f - std::pow(m->b1, (float)m->step), c2 = 1.f - std::pow(m->b2, (float)m->step);
-    k_adam<<<blocks(m->n_params, 256), 256, 0, st>>>((float*)m->P.p, (const float*)m->G.p, (float*)m->M.p,
-                                                     (float*)m->V.p, m->n_params, lr, m->b1, m->b2, m->eps, c1, c2,
-                                                     (__nv_bfloat16*)m->PH.p, (const unsigned char*)m->ISW.p);
-    MCK(cudaGetLastError());
+    MCK(launch_dep(k_adam, blocks(m->n_params, 256), 256, 0, st, (float*)m->P.p, (const float*)m->G.p, (float*)m->M.p,
+                   (float*)m->V.p, m->n_params, lr, m->b1, m->b2, m->eps, c1, c2, (__nv_bfloat16*)m->PH.p,
+                   (const unsigned char*)m->ISW.p));
     return MIRAGE_OK;
 }
 
@@ -624,17 +810,20 @@ int mirage_mlp_train(mirage_mlp_t* m, const float* x, const float* t, int n, int
     const long long s0 = m->step;
     MCK(cudaMemcpyAsync(dstep, &s0, sizeof(long long), cudaMemcpyHostToDevice, st));
 
-    // one training step: draw rows, forward, MSE gradient, Adam; captured once
+    const Draw draw{idx, (__nv_bfloat16*)m->A.p, x, batch, n, m->dims[0], seed};
+    const unsigned db = blocks((long)batch * m->dims[0], 256), nb = blocks(m->n_params, 256);
+    k_draw<<<db, 256, 0, st>>>(draw, dstep);
+    MCK(cudaGetLastError());
+
+    // one training step: forward, MSE gradient, Adam, the next step's rows;
+    // captured once
     cudaGraph_t graph = nullptr;
     MCK(cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeThreadLocal));
-    k_sample_rows<<<blocks(batch, 256), 256, 0, m->cap>>>(idx, batch, n, seed, dstep);
-    r = backward_pass(m, x, t, batch, y, false, m->cap, idx);
-    if (!r) {
-        k_adam_dev<<<blocks(m->n_params, 256), 256, 0, m->cap>>>(
-            (float*)m->P.p, (const float*)m->G.p, (float*)m->M.p, (float*)m->V.p, m->n_params, lr, m->b1, m->b2,
-            m->eps, dstep, (__nv_bfloat16*)m->PH.p, (const unsigned char*)m->ISW.p);
-        k_step_inc<<<1, 1, 0, m->cap>>>(dstep);
-    }
+    r = backward_pass(m, x, t, batch, y, false, m->cap, idx, dstep);
+    if (!r && launch_dep(k_adam_dev, nb + db, 256, 0, m->cap, (float*)m->P.p, (const float*)m->G.p, (float*)m->M.p,
+                         (float*)m->V.p, m->n_params, lr, m->b1, m->b2, m->eps, (const long long*)dstep,
+                         (__nv_bfloat16*)m->PH.p, (const unsigned char*)m->ISW.p, nb, draw) != cudaSuccess)
+        r = mlp_fail(MIRAGE_ERR_CUDA, "mlp_train: launch failed");
     const cudaError_t ec = cudaStreamEndCapture(m->cap, &graph);
     if (r) {
         if (graph) cudaGraphDestroy(graph);
