@@ -529,7 +529,7 @@ int upload(mirage_ctx* ctx, cudaStream_t st, std::initializer_list<UploadPart> p
 // CTAs per candidate trace and count, one CTA per candidate places)
 template <typename T>
 int launch_raytrace(mirage_ctx* ctx, const Prob<T>* dprobs, const int* dcand, const double* d_lens, int cand0,
-                    int n_cand, const CandScratch<T>& cs, long long max_cells, long long max_npix, cudaStream_t st);
+                    int n_cand, const CandScratch<T>& cs, long long max_cells, long long max_npix, long long max_rays, cudaStream_t st);
 
 #define TRY(x)                      \
     do {                            \
@@ -558,10 +558,28 @@ struct Stager {
 
 template <typename T>
 int launch_raytrace(mirage_ctx* ctx, const Prob<T>* dprobs, const int* dcand, const double* d_lens, int cand0,
-                    int n_cand, const CandScratch<T>& cs, long long max_cells, long long max_npix, cudaStream_t st) {
+                    int n_cand, const CandScratch<T>& cs, long long max_cells, long long max_npix, long long max_rays, cudaStream_t st) {
     constexpr int prec = prec_of<T>();
     const KernelTable& tb = table();
     const size_t cells_smem = (size_t)max_cells * 4;
+    // Ray numbers in shared memory: two launches (measured, one 64 x 64 candidate:
+    // 30 us against 260 for one CTA; 256 candidates: 0.3 against 0.53 ms).  The
+    // CTAs of the trace take at least RT_MIN_PIX pixels, and no more of them than
+    // fill the device twice
+    const size_t place_smem = sizeof(int) * (size_t)(max_cells + max_rays);
+    if (place_smem <= (size_t)ctx->max_smem - 2048 && n_cand <= 65535) {
+        constexpr long long RT_MIN_PIX = 32;
+        long long chunk_l = std::max(RT_MIN_PIX, (max_npix * n_cand + 16 * ctx->sm_count - 1) / (16 * ctx->sm_count));
+        int chunk = (int)std::min<long long>(chunk_l, RT_THREADS);
+        const long long per = std::max<long long>(1, std::min((max_npix + chunk - 1) / chunk, (16LL * ctx->sm_count + n_cand - 1) / n_cand));
+        int c0 = cand0;
+        CandScratch<T> csv = cs;
+        void* a1[] = {(void*)&dprobs, (void*)&dcand, (void*)&d_lens, &c0, &chunk, &csv};
+        TRY(launch(ctx, tb.rt_rays[prec], dim3((unsigned)per, n_cand), dim3(RT_THREADS), a1, 0, st));
+        TRY(set_smem(ctx, tb.rt_cells[prec], place_smem));
+        void* a2[] = {(void*)&dprobs, (void*)&dcand, (void*)&d_lens, &c0, &csv};
+        return launch(ctx, tb.rt_cells[prec], dim3(n_cand), dim3(RT_PLACE_THREADS), a2, place_smem, st);
+    }
     if (n_cand < ctx->sm_count && max_npix >= 128 * 128) {
         const int chunk = 2 * NTHREADS;
         const int n_chunks = (int)((max_npix + chunk - 1) / chunk);
@@ -1070,6 +1088,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     for (Group* g : glist) TRY(set_smem(ctx, g->fn, g->smem));
     if (spec_stride) TRY(set_smem(ctx, tb.psf_spectra[prec], fft_smem_bytes(1024)));
     TRY(set_smem(ctx, tb.raytrace[prec], (size_t)max_cells * 4));
+    if (4 * (max_cells + max_rays) <= ctx->max_smem - 2048) TRY(set_smem(ctx, tb.rt_cells[prec], sizeof(int) * (size_t)(max_cells + max_rays)));
     TRY(set_smem(ctx, tb.rt_place[prec], (size_t)max_cells * 4));
 
     CglsArgs<T> A;
@@ -1129,7 +1148,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         if (o.mode == MIRAGE_MODE_BATCHED) {
             if (timing) cudaEventRecord(ctx->ev[0], st);
             // 1) ray trace every candidate
-            rc = launch_raytrace<T>(ctx, dprobs, dcand, d_lens, 0, n_cand, cs, max_cells, max_npix, st);
+            rc = launch_raytrace<T>(ctx, dprobs, dcand, d_lens, 0, n_cand, cs, max_cells, max_npix, max_rays, st);
             if (rc) break;
             // 2) CGLS items, one persistent launch per kernel class
             if (cudaMemsetAsync(dcnt, 0, sizeof(int) * n_counters, st) != cudaSuccess) {
@@ -1242,7 +1261,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                 }
                 TRY(set_smem(ctx, fn, item_smem));
                 int cand0 = c, nc = 1;
-                rc = launch_raytrace<T>(ctx, dprobs, dcand, d_lens, c, 1, cs, max_cells, max_npix, st);
+                rc = launch_raytrace<T>(ctx, dprobs, dcand, d_lens, c, 1, cs, max_cells, max_npix, max_rays, st);
                 if (rc) break;
                 A.items = ditems + plain_off[c];
                 A.n_items = plain_off[c + 1] - plain_off[c];
@@ -1357,7 +1376,6 @@ int forward_impl(mirage_ctx* ctx, const mirage_problem_t* prob, const double* le
     CandScratch<T> cs;
     fill_scratch<T>(cs, ctx, true, sE, sInv, sCst, sPad);
     const KernelTable& tb = table();
-    TRY(launch_raytrace<T>(ctx, dprob, dcand, lens, 0, 1, cs, P.ncells, (long long)P.npix, st));
     if constexpr (sizeof(T) == 4) {
         // banded kernel: taps as kernel parameters, L s gathered into shared memory
         const void* fb = (P.Np == 1 && P.interp != MIRAGE_INTERP_BICUBIC && P.K < MAX_K && P.K * P.K <= MAX_FTAP)
@@ -1367,20 +1385,28 @@ int forward_impl(mirage_ctx* ctx, const mirage_problem_t* prob, const double* le
             const int bt = std::min(FWD_THREADS / P.tiles_x, P.tiles_y);
             const size_t smb = fwd_band_smem(P, bt);
             if ((long long)smb <= ctx->max_smem) {
-                TRY(ctx->fpix.ensure(sizeof(float4) * (size_t)P.npix));
+                // the rays in pixel order are all that this kernel reads: no
+                // placement by cells
+                const int chunk = (int)std::min<long long>(RT_THREADS, std::max(32LL, (P.npix + 8LL * ctx->sm_count - 1) / (8LL * ctx->sm_count)));
+                const int n_rays_cta = (P.npix + chunk - 1) / chunk;
+                const size_t pix_bytes = (sizeof(float4) * (size_t)P.npix + 15) / 16 * 16;
+                TRY(ctx->fpix.ensure(pix_bytes + sizeof(int) * (size_t)n_rays_cta));
                 float4* pm = ctx->fpix.as<float4>();
+                int* flags = reinterpret_cast<int*>(ctx->fpix.as<char>() + pix_bytes);
                 {
                     CandScratch<float> csv = cs;
                     const Prob<float>* dp0 = dprob;
-                    void* ap[] = {(void*)&dp0, &csv, (void*)&pm};
-                    TRY(launch(ctx, tb.pixmap, dim3(std::min((P.npix + NTHREADS - 1) / NTHREADS, 4 * ctx->sm_count)),
-                               dim3(NTHREADS), ap, 0, st));
+                    int ch = chunk;
+                    void* ap[] = {(void*)&dp0, (void*)&lens, &csv, (void*)&pm, (void*)&flags, &ch};
+                    TRY(launch(ctx, tb.fwd_rays, dim3(n_rays_cta), dim3(RT_THREADS), ap, 0, st));
                 }
                 std::vector<unsigned char> fab(sizeof(FwdArgs), 0);
                 FwdArgs* fa = reinterpret_cast<FwdArgs*>(fab.data());
                 fa->probs = dprob;
                 fa->cs = cs;
                 fa->pixmap = pm;
+                fa->flags = flags;
+                fa->n_flags = n_rays_cta;
                 fa->S = reinterpret_cast<const float*>(s);
                 fa->n_src = n_src;
                 fa->model = reinterpret_cast<float*>(model);
@@ -1394,6 +1420,7 @@ int forward_impl(mirage_ctx* ctx, const mirage_problem_t* prob, const double* le
             }
         }
     }
+    TRY(launch_raytrace<T>(ctx, dprob, dcand, lens, 0, 1, cs, P.ncells, (long long)P.npix, (long long)P.nrays, st));
     const void* fn = pick_fwd(prec, P.K);
     const size_t smem = align_up<T>(sizeof(T) * P.K * P.kp, 16) + 2 * 33 * sizeof(double) + 16;
     TRY(set_smem(ctx, fn, smem));
@@ -1475,7 +1502,7 @@ int iter_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     const Prob<T>* dprobs = ctx->probs.as<Prob<T>>();
     const int* dcand = ctx->cand_prob.as<int>();
     const KernelTable& tb = table();
-    TRY(launch_raytrace<T>(ctx, dprobs, dcand, lens, 0, n_cand, cs, max_cells, max_npix, st));
+    TRY(launch_raytrace<T>(ctx, dprobs, dcand, lens, 0, n_cand, cs, max_cells, max_npix, max_rays, st));
     const void* fn = (k_all > 0 && k_all < MAX_K && tb.iter[prec][k_all]) ? tb.iter[prec][k_all] : tb.iter[prec][0];
     TRY(set_smem(ctx, fn, smem));
     IterArgs<T> A;

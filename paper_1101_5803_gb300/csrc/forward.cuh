@@ -6,7 +6,7 @@
 // processed in bands of whole tile rows (two buffers: one band is filled
 // while the previous one is convolved), each band's zero-padded L s values
 // (its rows plus the K-1 halo rows) gathered straight into shared memory
-// from a pixel-ordered map of the rays' cells and weights (k_pixmap), so
+// from a pixel-ordered map of the rays' cells and weights (k_fwd_rays), so
 // L s never goes to global memory.  Each thread owns one 4x4 tile of the
 // band and convolves it with the PSF taps (staged in shared memory, read as
 // warp-uniform broadcasts), in a loop over pairs of tap rows (each input row is loaded once per pair; the
@@ -25,6 +25,8 @@ struct FwdArgs {
     const Prob<float>* probs;
     CandScratch<float> cs;
     const float4* pixmap;  // [npix] {cell base (int bits) or -1, u, v, 0} in pixel order
+    const int* flags;      // [n_flags] of k_fwd_rays' CTAs: 1 = has active pixels, 2 = invalid lens
+    int n_flags;
     const float* S;   // [n_src][ns]
     int n_src;
     float* model;     // nullable [n_src][npix]
@@ -40,20 +42,42 @@ __host__ inline size_t fwd_band_smem(const Prob<float>& P, int band_tiles) {
            2 * sizeof(float) * (size_t)(band_tiles * TILE + P.K - 1) * P.Wp;
 }
 
-// pixel-ordered ray map of candidate 0 (one ray per pixel)
+// The lens's rays in pixel order (one ray per pixel), sqrt(W) and the padded
+// data: what the banded kernel reads.  `chunk` pixels per CTA, small enough to
+// spread the FP64 trace over the device.  (A call on one 64 x 64 source: 282 us
+// with one CTA tracing and sorting the rays by cell, as the solves need them, and
+// this map read back from that; 91 us with the sort spread out; 55 us without.)
 template <int UNUSED = 0>
-__global__ void __launch_bounds__(NTHREADS) k_pixmap(const Prob<float>* __restrict__ probs, CandScratch<float> cs,
-                                                   float4* __restrict__ pixmap) {
+__global__ void __launch_bounds__(RT_THREADS) k_fwd_rays(const Prob<float>* __restrict__ probs,
+                                                         const double* __restrict__ lens, CandScratch<float> cs,
+                                                         float4* __restrict__ pixmap, int* __restrict__ flags, int chunk) {
     const Prob<float>& P = probs[0];
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < P.npix; j += gridDim.x * blockDim.x) {
-        const int e = cs.inv[j];
-        float4 m = make_float4(__int_as_float(-1), 0.f, 0.f, 0.f);
-        if (e >= 0) {
-            const Entry<float> en = cs.E[e];
-            m = make_float4(__int_as_float(en.base), en.u, en.v, 0.f);
+    const LensT<double> L = make_lens<double>(lens);
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.plen; i += gridDim.x * blockDim.x) {  // the zero frame
+        const int yp = i / P.Wp, y = yp - P.hk, x = i - yp * P.Wp - P.xoff;
+        if (L.bad || x < 0 || x >= P.nx || y < 0 || y >= P.ny) {
+            cs.swp[i] = 0.f;
+            cs.dpad[i] = 0.f;
         }
-        pixmap[j] = m;
     }
+    int active = 0;
+    if (!L.bad) {
+        const int j1 = min((int)(blockIdx.x + 1) * chunk, P.npix);
+        for (int j = blockIdx.x * chunk + threadIdx.x; j < j1; j += blockDim.x) {
+            const int y = j / P.nx, x = j - y * P.nx;
+            int base;
+            double u, v;
+            const bool any = rt_ray(P, L, x, y, 0, base, u, v);
+            pixmap[j] = make_float4(__int_as_float(base), (float)u, (float)v, 0.f);
+            const float w = (any && P.mask[j]) ? 1.f / P.sigma[j] : 0.f;
+            const int pp = (y + P.hk) * P.Wp + x + P.xoff;
+            cs.swp[pp] = w;
+            cs.dpad[pp] = P.d[j];
+            active |= w != 0.f;
+        }
+    }
+    active = __syncthreads_or(active);
+    if (threadIdx.x == 0) flags[blockIdx.x] = L.bad ? 2 : (active != 0);
 }
 
 // One 4x4 output tile: out[r][c] = sum_{a,b} t[a][b] in[r + a][c + b + SHF]
@@ -120,7 +144,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) k_forward_band(const __grid_co
     extern __shared__ __align__(16) unsigned char smem[];
     const Prob<float>& P = FA.probs[0];
     const CandScratch<float>& cs = FA.cs;
-    const Geo<float> g = geo_of(P, cs.nent[0]);
+    const Geo<float> g = geo_of(P, 0);  // (the ray count is not used)
     double* red = reinterpret_cast<double*>(smem + 16);
     float* taps = reinterpret_cast<float*>(smem + 16 + 2 * 33 * sizeof(double));
     float* s_sh = taps + align_up<float>(K * K, 4);
@@ -135,8 +159,13 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) k_forward_band(const __grid_co
     const int tiles_y = g.ntiles / g.tiles_x;
     const int n_bands = (tiles_y + BT - 1) / BT;
     const int rows = BR + K - 1;  // band rows in the buffer
-    if (blockIdx.x == 0 && tid == 0 && FA.status) FA.status[0] = cs.cstat[0];
-    const bool bad = (cs.cstat[0] & ST_BADPARAM) != 0;
+    const bool bad = FA.flags[0] == 2;
+    if (blockIdx.x == 0 && FA.status) {
+        int some = 0;
+        for (int i = tid; i < FA.n_flags; i += bs) some |= FA.flags[i];
+        some = __syncthreads_or(some);
+        if (tid == 0) FA.status[0] = bad ? ST_BADPARAM : some ? 0 : ST_EMPTY;
+    }
     int which = 0;
     for (int k = blockIdx.x; k < FA.n_src; k += gridDim.x) {
         __syncthreads();

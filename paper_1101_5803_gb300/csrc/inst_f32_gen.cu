@@ -16,6 +16,8 @@ void fill_f32_gen(KernelTable& t) {
     t.rt_place[0] = (const void*)k_rt_place<float>;
     t.rt_scatter[0] = (const void*)k_rt_scatter<float>;
     t.rt_sortcells[0] = (const void*)k_rt_sortcells<float>;
+    t.rt_rays[0] = (const void*)k_rt_rays<float>;
+    t.rt_cells[0] = (const void*)k_rt_cells<float>;
     t.finalize[0] = (const void*)k_finalize<float>;
     t.psf_spectra[0] = (const void*)k_psf_spectra<float>;
 }

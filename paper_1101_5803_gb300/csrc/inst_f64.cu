@@ -13,6 +13,8 @@ void fill_f64(KernelTable& t) {
     t.rt_place[1] = (const void*)k_rt_place<double>;
     t.rt_scatter[1] = (const void*)k_rt_scatter<double>;
     t.rt_sortcells[1] = (const void*)k_rt_sortcells<double>;
+    t.rt_rays[1] = (const void*)k_rt_rays<double>;
+    t.rt_cells[1] = (const void*)k_rt_cells<double>;
     t.finalize[1] = (const void*)k_finalize<double>;
     t.psf_spectra[1] = (const void*)k_psf_spectra<double>;
 }

@@ -225,53 +225,63 @@ static_assert(sizeof(CgCtl) <= 128, "CG control block must fit its reserved shar
 //   rt_trace_pixels : trace the rays of image pixels [j0, j1) (this CTA's
 //                     threads), write them in ray order, sqrt(W) and the
 //                     padded data, and count rays per cell into `counts`
-//                     and active pixels into `active` (shared or global);
+//                     and active pixels into `active` (shared or global, or
+//                     null: not counted);
 //   rt_place        : scan the cell counts and place the rays sorted by
 //                     cell, stable within a cell (one warp, in ray order).
 // Rays are traced in FP64 whatever T is: the refinement residual uses these
 // weights, and FP32-rounded weights would perturb the operator by ~1e-7,
 // which the conditioning of small-lambda systems amplifies.
 // ---------------------------------------------------------------------------
+// one (sub-)pixel ray: its cell's base source pixel and offsets, or -1 and
+// false when it misses the source grid
+template <typename T>
+__device__ __forceinline__ bool rt_ray(const Prob<T>& P, const LensT<double>& L, int x, int y, int a, int& base,
+                                       double& u, double& v) {
+    const double half_x = 0.5 * (double)(P.nx - 1), half_y = 0.5 * (double)(P.ny - 1);
+    const double fxmax = (double)(P.sx - 1), fymax = (double)(P.sy - 1);
+    const double tx = P.cx + ((double)x - half_x) * P.pix;
+    const double ty = P.cy + ((double)y - half_y) * P.pix;
+    const int ax = a % P.n_sub, ay = a / P.n_sub;
+    double bx, by;
+    trace_ray(L, tx + P.sub0 + (double)ax * P.subd, ty + P.sub0 + (double)ay * P.subd, bx, by);
+    const double fx = (bx - P.c0x) / P.hx;
+    const double fy = (by - P.c0y) / P.hy;
+    base = -1;
+    u = v = 0;
+    if (!((fx >= 0.0) && (fx <= fxmax) && (fy >= 0.0) && (fy <= fymax))) return false;
+    const int ix0 = min((int)m_floor(fx), P.sx - 2);
+    const int iy0 = min((int)m_floor(fy), P.sy - 2);
+    base = iy0 * P.sx + ix0;
+    u = fx - (double)ix0;
+    v = fy - (double)iy0;
+    if (P.interp == 1) {  // nearest centre: the one-hot bilinear weights
+        u = u >= 0.5 ? 1.0 : 0.0;
+        v = v >= 0.5 ? 1.0 : 0.0;
+    }
+    return true;
+}
+
 template <typename T>
 __device__ __forceinline__ void rt_trace_pixels(const Prob<T>& P, const LensT<double>& L, const CandScratch<T>& cs,
                                                 int c, int j0, int j1, int* counts, int* active) {
     Entry<double>* Et = cs.Etmp + (long long)c * cs.sE;
     T* swp = cs.swp + (long long)c * cs.sPad;
     T* dpad = cs.dpad + (long long)c * cs.sPad;
-    const double half_x = 0.5 * (double)(P.nx - 1), half_y = 0.5 * (double)(P.ny - 1);
-    const double fxmax = (double)(P.sx - 1), fymax = (double)(P.sy - 1);
     int my_active = 0;
     for (int j = j0 + (int)threadIdx.x; j < j1; j += blockDim.x) {
         const int x = j % P.nx, y = j / P.nx;
-        const double tx = P.cx + ((double)x - half_x) * P.pix;
-        const double ty = P.cy + ((double)y - half_y) * P.pix;
         const int pp = (y + P.hk) * P.Wp + x + P.xoff;
         bool any = false;
         for (int a = 0; a < P.Np; ++a) {
-            const int ax = a % P.n_sub, ay = a / P.n_sub;
-            double bx, by;
-            trace_ray(L, tx + P.sub0 + (double)ax * P.subd, ty + P.sub0 + (double)ay * P.subd, bx, by);
-            const double fx = (bx - P.c0x) / P.hx;
-            const double fy = (by - P.c0y) / P.hy;
-            const bool m = (fx >= 0.0) && (fx <= fxmax) && (fy >= 0.0) && (fy <= fymax);
             Entry<double> e;
             e.ppos = pp;
-            if (m) {
-                const int ix0 = min((int)m_floor(fx), P.sx - 2);
-                const int iy0 = min((int)m_floor(fy), P.sy - 2);
-                e.base = iy0 * P.sx + ix0;
-                e.u = fx - (double)ix0;
-                e.v = fy - (double)iy0;
-                if (P.interp == 1) {  // nearest centre: the one-hot bilinear weights
-                    e.u = e.u >= 0.5 ? 1.0 : 0.0;
-                    e.v = e.v >= 0.5 ? 1.0 : 0.0;
+            if (rt_ray(P, L, x, y, a, e.base, e.u, e.v)) {
+                if (counts) {
+                    const int iy0 = e.base / P.sx;
+                    atomicAdd(&counts[iy0 * P.ncx + (e.base - iy0 * P.sx)], 1);
                 }
-                atomicAdd(&counts[iy0 * P.ncx + ix0], 1);
                 any = true;
-            } else {
-                e.base = -1;
-                e.u = 0;
-                e.v = 0;
             }
             Et[(long long)j * P.Np + a] = e;
         }
@@ -280,7 +290,7 @@ __device__ __forceinline__ void rt_trace_pixels(const Prob<T>& P, const LensT<do
         dpad[pp] = P.d[j];
         my_active += (w != (T)0);
     }
-    if (my_active) atomicAdd(active, my_active);
+    if (my_active && active) atomicAdd(active, my_active);
 }
 
 // sh_counts: [ncells] shared memory holding the cell counts on entry;
@@ -425,6 +435,157 @@ __global__ void __launch_bounds__(NTHREADS) k_raytrace(const Prob<T>* __restrict
     rt_trace_pixels(P, L, cs, c, 0, P.npix, sh_counts, &s_active);
     __syncthreads();
     rt_place(P, cs, c, sh_counts, s_chunk, s_active);
+}
+
+// ---------------------------------------------------------------------------
+// Ray trace in two launches, for problems whose ray numbers fit in shared
+// memory: k_rt_rays traces the rays of all candidates on as many CTAs as the
+// device holds (about 150 FP64 operations a ray at 2 a clock and SM bound it:
+// one CTA took 0.25 ms for the 4096 rays of a 64 x 64 image), and k_rt_cells
+// places them, one CTA of 1024 threads per candidate: cell counts, scan, ray
+// numbers scattered to their cells and each cell sorted back into ray order in
+// shared memory, then one pass over the rays.  The same arrays as k_raytrace.
+// ---------------------------------------------------------------------------
+constexpr int RT_THREADS = 128, RT_PLACE_THREADS = 1024;
+
+template <typename T>
+__global__ void __launch_bounds__(RT_THREADS) k_rt_rays(const Prob<T>* __restrict__ probs,
+                                                        const int* __restrict__ cand_prob,
+                                                        const double* __restrict__ lens, int cand0, int chunk,
+                                                        CandScratch<T> cs) {
+    const int c = cand0 + blockIdx.y;
+    const Prob<T>& P = probs[cand_prob[c]];
+    const LensT<double> L = make_lens<double>(lens + 7LL * c);
+    T* swp = cs.swp + (long long)c * cs.sPad;
+    T* dpad = cs.dpad + (long long)c * cs.sPad;
+    // the zero frame (everything for an invalid lens)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.plen; i += gridDim.x * blockDim.x) {
+        const int yp = i / P.Wp, y = yp - P.hk, x = i - yp * P.Wp - P.xoff;
+        if (L.bad || x < 0 || x >= P.nx || y < 0 || y >= P.ny) {
+            swp[i] = 0;
+            dpad[i] = 0;
+        }
+    }
+    if (L.bad) return;
+    for (int j0 = blockIdx.x * chunk; j0 < P.npix; j0 += gridDim.x * chunk)
+        rt_trace_pixels(P, L, cs, c, j0, min(j0 + chunk, P.npix), (int*)nullptr, (int*)nullptr);
+}
+
+// shared memory of k_rt_cells: cell starts, then ray numbers
+template <typename T>
+__host__ inline size_t rt_cells_smem(const Prob<T>& P) {
+    return sizeof(int) * ((size_t)P.ncells + (size_t)P.nrays);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(RT_PLACE_THREADS) k_rt_cells(const Prob<T>* __restrict__ probs,
+                                                               const int* __restrict__ cand_prob,
+                                                               const double* __restrict__ lens, int cand0,
+                                                               CandScratch<T> cs) {
+    const int c = cand0 + blockIdx.x;
+    const Prob<T>& P = probs[cand_prob[c]];
+    extern __shared__ int sh_counts[];  // [ncells] counts, then ends; [nrays] ray numbers by cell
+    __shared__ int s_warp[RT_PLACE_THREADS / 32], s_active;
+    int* list = sh_counts + P.ncells;
+    const int tid = threadIdx.x, lane = tid & 31, bs = RT_PLACE_THREADS;
+    if (make_lens<double>(lens + 7LL * c).bad) {
+        rt_bad(P, cs, c);
+        return;
+    }
+    const Entry<double>* Et = cs.Etmp + (long long)c * cs.sE;
+    Entry<T>* E = cs.E + (long long)c * cs.sE;
+    Entry<double>* E64 = cs.E64 + (long long)c * cs.sE;
+    int* inv = cs.inv + (long long)c * cs.sInv;
+    int* cst = cs.cst + (long long)c * cs.sCst;
+    const T* swp = cs.swp + (long long)c * cs.sPad;
+    for (int i = tid; i < P.ncells; i += bs) sh_counts[i] = 0;
+    if (tid == 0) s_active = 0;
+    __syncthreads();
+    auto cell_of = [&](int base) {
+        const int iy0 = base / P.sx;
+        return iy0 * P.ncx + (base - iy0 * P.sx);
+    };
+    for (int r = tid; r < P.nrays; r += bs) {
+        const int base = Et[r].base;
+        if (base >= 0) atomicAdd(&sh_counts[cell_of(base)], 1);
+    }
+    bool active = false;
+    for (int i = tid; i < P.plen; i += bs) active |= swp[i] != (T)0;
+    if (__any_sync(0xffffffffu, active) && lane == 0) s_active = 1;
+    __syncthreads();
+    // exclusive scan: a run of cells per thread, then warp and block sums
+    const int chunk = (P.ncells + bs - 1) / bs;
+    const int lo = min(tid * chunk, P.ncells), hi = min(lo + chunk, P.ncells);
+    int sum = 0;
+    for (int i = lo; i < hi; ++i) sum += sh_counts[i];
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+    }
+    if (lane == 31) s_warp[tid >> 5] = inc;
+    __syncthreads();
+    if (tid < 32) {
+        const int v = s_warp[tid];
+        int w = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        s_warp[tid] = w - v;
+        if (tid == 31) {
+            cst[P.ncells] = w;
+            cs.nent[c] = w;
+            cs.cstat[c] = s_active ? 0 : ST_EMPTY;
+        }
+    }
+    __syncthreads();
+    int run = s_warp[tid >> 5] + inc - sum;
+    for (int i = lo; i < hi; ++i) {
+        const int v = sh_counts[i];
+        sh_counts[i] = run;
+        cst[i] = run;
+        run += v;
+    }
+    __syncthreads();
+    for (int r = tid; r < P.nrays; r += bs) {
+        const int base = Et[r].base;
+        if (base >= 0)
+            list[atomicAdd(&sh_counts[cell_of(base)], 1)] = r;  // (starts become ends)
+        else
+            inv[r] = -1;
+    }
+    __syncthreads();
+    for (int i = tid; i < P.ncells; i += bs) {  // insertion sort (cells hold few rays)
+        const int k0 = i > 0 ? sh_counts[i - 1] : 0, k1 = sh_counts[i];
+        for (int a = k0 + 1; a < k1; ++a) {
+            const int key = list[a];
+            int b = a - 1;
+            while (b >= k0 && list[b] > key) {
+                list[b + 1] = list[b];
+                --b;
+            }
+            list[b + 1] = key;
+        }
+    }
+    __syncthreads();
+    const int n = P.ncells > 0 ? sh_counts[P.ncells - 1] : 0;
+    for (int p = tid; p < n; p += bs) {
+        const int r = list[p];
+        const Entry<double> e = Et[r];
+        E64[p] = e;
+        if ((void*)E != (void*)E64) {
+            Entry<T> et;
+            et.ppos = e.ppos;
+            et.base = e.base;
+            et.u = (T)e.u;
+            et.v = (T)e.v;
+            E[p] = et;
+        }
+        inv[r] = p;
+    }
 }
 
 // ---------------------------------------------------------------------------

@@ -16,6 +16,8 @@ struct KernelTable {
     const void* rt_place[2];  //                  scan and place (one CTA per candidate)
     const void* rt_scatter[2];    // parallel placement, one ray per pixel
     const void* rt_sortcells[2];
+    const void* rt_rays[2];   // two-launch ray trace: trace (many CTAs per candidate)
+    const void* rt_cells[2];  //                       place (one CTA per candidate)
     const void* finalize[2];
     // fast[K][v][mode]: two-CTA-per-SM FP32 kernel, v = 0 for ns <= 1024,
     // 1 for ns <= 2304; mode = tap source (0 shared, 1 params FFMA, 2 params
@@ -25,7 +27,7 @@ struct KernelTable {
     const void* iter[2][MAX_K];
     // fwdb[K]: banded FP32 forward batch (one ray per pixel)
     const void* fwdb[MAX_K];
-    const void* pixmap;  // pixel-ordered ray map for the banded forward batch
+    const void* fwd_rays;  // pixel-ordered rays for the banded forward batch
     const void* psf_spectra[2];  // PSF spectra of the FFT-convolution problems
     // cluster[K][nt]: general kernel on a thread-block cluster (FP32), nt = 0
     // for 256 threads a CTA, 1 for 512
