@@ -873,9 +873,18 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         }
         chain_budget = tw / (double)cgls_slots(ctx, 2);
     }
+    long long n_items = 0;
+    for (int c = 0; c < n_cand; ++c) n_items += n_lam[c];
     for (int c = 0; c < n_cand; ++c) {
         const Prob<T>& P = hp[prob_idx[c]];
-        const int place = pick_place<T>(ctx, P, o.place);
+        int place = pick_place<T>(ctx, P, o.place);
+        // FP64, everything in shared memory: two CTAs per SM (128 registers a
+        // thread) where two fit and there are many items a slot.  At 32 x 32, 256
+        // candidates x 10 lambdas took 159 ms with two and 191 with one, 64
+        // candidates 55.5 and 48.9: with few items the longest one's time counts
+        if (sizeof(T) == 8 && place == PLACE_SMEM && o.place == 0 && o.mode == MIRAGE_MODE_BATCHED &&
+            n_items >= 8LL * ctx->sm_count && 2 * ((long long)smem_bytes<T>(P, PLACE_SMEM) + 1024) <= ctx->max_smem_sm)
+            place = PLACE_SMEM2;
         const bool big = place != PLACE_SMEM;
         const void* fn = pick_cgls(prec, place, P.fft_m ? 0 : P.K);
         size_t item_smem = smem_bytes<T>(P, layout_of(place));

@@ -1154,6 +1154,37 @@ __device__ __forceinline__ void st4(double* p, const V4<double>& o) {
 
 enum : int { CONV_Q = 0, CONV_RAW = 1 };
 
+// FP64 convolution of one row of four output pixels: out[c] = sum_{a,b}
+// taps[a][b] Pb[a Wp + c + b + sh], terms in the order a, b.  Small images have
+// fewer 4 x 4 tiles than a CTA has threads (64 of 256 at 32 x 32), and the FP64
+// units of the idle warps' SM sub-partitions would stand still; a row a thread
+// keeps them all busy.
+__device__ __forceinline__ void conv_row64(const double* __restrict__ Pb, int Wp, const double* __restrict__ taps, int K,
+                                           int KP, double (&acc)[TILE]) {
+#pragma unroll
+    for (int c = 0; c < TILE; ++c) acc[c] = 0.0;
+    for (int a = 0; a < K; ++a) {
+        const double* row = Pb + a * Wp;
+        double w[TILE];
+#pragma unroll
+        for (int c = 0; c < TILE - 1; ++c) w[c + 1] = row[c];
+#pragma unroll 5
+        for (int b = 0; b < K; ++b) {  // sliding window of four inputs
+#pragma unroll
+            for (int c = 0; c < TILE - 1; ++c) w[c] = w[c + 1];
+            w[TILE - 1] = row[b + TILE - 1];
+            const double t = taps[a * KP + b];
+#pragma unroll
+            for (int c = 0; c < TILE; ++c) acc[c] = fma(t, w[c], acc[c]);
+        }
+    }
+}
+// whether an image is convolved by rows
+template <typename T>
+__device__ __forceinline__ bool conv_by_rows(const Geo<T>& g) {
+    return sizeof(T) == 8 && 2 * g.ntiles <= (int)blockDim.x;
+}
+
 // One convolution over all owned tiles (one non-inlined copy of the
 // unrolled tile code per kernel):
 //   CONV_Q   : dst = sqrt(W) * conv, returns sum dst^2
@@ -1162,6 +1193,32 @@ template <typename T, int K, bool SH>
 __device__ __noinline__ T conv_pass(const T* __restrict__ src, const T* __restrict__ taps,
                                          const T* __restrict__ swp, T* __restrict__ dst, Geo<T> g, int mode) {
     T ss = 0;
+    if constexpr (sizeof(T) == 8) {
+        if (conv_by_rows(g)) {
+            const int kk = K > 0 ? K : g.K, kp = K > 0 ? (K + 3) & ~3 : g.kp;
+            for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
+                const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
+                double acc[TILE];
+                conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, kk, kp, acc);
+                const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
+#pragma unroll
+                for (int c = 0; c < TILE; ++c) dst[pp + c] = mode == CONV_Q ? swp[pp + c] * acc[c] : acc[c];
+            }
+            if (mode == CONV_Q) {  // the sum in the order of the tiles' owners
+                __syncthreads();
+                for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
+                    const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
+#pragma unroll
+                    for (int r = 0; r < TILE; ++r) {
+                        const V4<T> o = ld4(dst + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) ss = fma(o.v[c], o.v[c], ss);
+                    }
+                }
+            }
+            return ss;
+        }
+    }
     for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
         const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
         T acc[TILE][TILE];
@@ -1217,6 +1274,40 @@ __device__ __noinline__ double conv64_pass(const Work<T> w, Geo<T> g, int mode) 
     }
     const double* src = mode == 0 ? w.Pa : w.Pb;
     const double* taps = w.taps64 + (mode == 0 ? 0 : g.K * g.kp);
+    if (sizeof(T) == 8 && conv_by_rows(g)) {  // (Pc holds the residuals until their sum is taken)
+        for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
+            const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
+            double acc[TILE];
+            conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, g.K, g.kp, acc);
+            const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
+#pragma unroll
+            for (int c = 0; c < TILE; ++c) {
+                if (mode == 0) {
+                    const double sw = (double)w.swp[pp + c];
+                    const double res = sw * ((double)w.dpad[pp + c] - acc[c]);
+                    w.rimg[pp + c] = (T)res;
+                    w.Pb[pp + c] = sw * res;
+                    w.Pc[pp + c] = res;
+                } else {
+                    w.Pc[pp + c] = acc[c];
+                }
+            }
+        }
+        if (mode == 0) {
+            __syncthreads();
+            for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
+                const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
+#pragma unroll
+                for (int r = 0; r < TILE; ++r) {
+                    const V4<double> o = ld4(w.Pc + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) ss += o.v[c] * o.v[c];
+                }
+            }
+            __syncthreads();
+        }
+        return ss;
+    }
     for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
         const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
         double acc[TILE][TILE];
@@ -1421,13 +1512,15 @@ __host__ __device__ inline size_t align_up(size_t v, size_t a) {
 constexpr double FINAL_MARGIN = 0.8, FINAL_MARGIN64 = 0.3, MAX_TARGET = 0.5;
 
 enum : int { PLACE_SMEM = 0, PLACE_GLOBAL = 1, PLACE_MID = 2 };
-// kernel-table indices of the global-slab and split kernels compiled for two
+// kernel-table indices of the global-slab, split and shared kernels compiled for two
 // CTAs per SM (their buffers are laid out as PLACE_GLOBAL and PLACE_MID)
-constexpr int PLACE_GLOBAL2 = 3, PLACE_MID2 = 4;
+constexpr int PLACE_GLOBAL2 = 3, PLACE_MID2 = 4, PLACE_SMEM2 = 5;
 __host__ __device__ constexpr int layout_of(int place) {
-    return place == PLACE_GLOBAL2 ? PLACE_GLOBAL : place == PLACE_MID2 ? PLACE_MID : place;
+    return place == PLACE_GLOBAL2 ? PLACE_GLOBAL : place == PLACE_MID2 ? PLACE_MID : place == PLACE_SMEM2 ? PLACE_SMEM : place;
 }
-__host__ __device__ constexpr bool two_per_sm(int place) { return place == PLACE_GLOBAL2 || place == PLACE_MID2; }
+__host__ __device__ constexpr bool two_per_sm(int place) {
+    return place == PLACE_GLOBAL2 || place == PLACE_MID2 || place == PLACE_SMEM2;
+}
 
 template <typename T>
 __host__ __device__ inline size_t smem_bytes(const Prob<T>& P, int place) {
