@@ -35,6 +35,17 @@ struct CxOf<double> {
 
 constexpr int FFT_BUF_BYTES = 64 * 1024;  // shared ping-pong buffers of one batch
 
+// Single-precision convolutions on 64 x 64 and 128 x 128 grids keep the whole
+// half spectrum in shared memory (fftshared.cuh): rows of M + 1 points, and
+// one exchange buffer of M + M / 16 points for each of the 256 threads' transforms
+__host__ __device__ constexpr bool fft_shared(int M) { return M == 64 || M == 128; }
+// batch buffers of size-M plans (bytes), for CTAs of 256 threads
+__host__ __device__ constexpr int fft_buf_bytes(int M) {
+    return fft_shared(M) && 8 * ((M / 2 + 1) * (M + 1) + 256 * 16 / M * (M + M / 16)) > FFT_BUF_BYTES
+               ? 8 * ((M / 2 + 1) * (M + 1) + 256 * 16 / M * (M + M / 16))
+               : FFT_BUF_BYTES;
+}
+
 template <typename R>
 struct FftPlan {
     using C = typename CxOf<R>::type;
@@ -56,7 +67,7 @@ __host__ __device__ inline int fft_size_for(int n) {
 // shared bytes of the FFT path for size M: two plans, both twiddle tables
 // (with alignment slack) and the batch buffers
 __host__ __device__ inline size_t fft_smem_bytes(int M) {
-    return 128 + (size_t)(M - 1) * (sizeof(float2) + sizeof(double2)) + 64 + FFT_BUF_BYTES;
+    return 128 + (size_t)(M - 1) * (sizeof(float2) + sizeof(double2)) + 64 + fft_buf_bytes(M);
 }
 
 // transforms per batch for element type C

@@ -22,6 +22,7 @@
 
 #include "dfloat.cuh"
 #include "fftconv.cuh"
+#include "fftshared.cuh"
 #include "interp.cuh"
 #include "lcurve.cuh"
 #include "lens.cuh"
@@ -1349,6 +1350,24 @@ __device__ __noinline__ T conv_pass_fft(const FftPlan<T>* f, const T* __restrict
             dst[pp] = v;
         }
     };
+    if constexpr (sizeof(T) == 4) {
+        if (fft_shared(f->M) && blockDim.x == 256) {
+            auto put = [&](int y, int n, float v) {
+                const int pp = (y + g.hk) * g.Wp + n + g.xoff;
+                dst[pp] = mode == CONV_Q ? swp[pp] * v : v;
+            };
+            if (f->M == 64)
+                fft_convolve_shared<64>(*f, load, g.ny, put, g.ny, g.nx, mode != CONV_Q);
+            else
+                fft_convolve_shared<128>(*f, load, g.ny, put, g.ny, g.nx, mode != CONV_Q);
+            if (mode == CONV_Q)
+                fft_store_order(f->M, [&](int y, int n) {
+                    const float o = dst[(y + g.hk) * g.Wp + n + g.xoff];
+                    ss = fma(o, o, ss);
+                }, g.ny, g.nx);
+            return ss;
+        }
+    }
     fft_convolve<T>(*f, load, g.ny, store, g.ny, g.nx, mode != CONV_Q);
     return ss;
 }
