@@ -9,9 +9,11 @@
 // from a pixel-ordered map of the rays' cells and weights (k_fwd_rays), so
 // L s never goes to global memory.  Each thread owns one 4x4 tile of the
 // band and convolves it with the PSF taps (staged in shared memory, read as
-// warp-uniform broadcasts), in a loop over pairs of tap rows (each input row is loaded once per pair; the
-// loop body stays small enough for the instruction cache, which the fully
-// unrolled 21x21 tile is not).  chi^2: FP32 per tile, FP64 across tiles.
+// warp-uniform broadcasts), in a loop over two or three tap rows held in
+// registers (each input row is loaded once for them; the loop body stays small
+// enough for the instruction cache, which the fully unrolled 21x21 tile is
+// not).  chi^2: FP32 per tile, FP64 across tiles.  A population of 1024 sources
+// at 256 x 256 and K = 21: 1.89 -> 1.61 ms against one load per tap.
 #pragma once
 
 #include "fast.cuh"
@@ -37,7 +39,7 @@ struct FwdArgs {
 
 // shared memory: taps, source vector, then two bands of (band rows + K - 1) x Wp
 __host__ inline size_t fwd_band_smem(const Prob<float>& P, int band_tiles) {
-    return 16 + 2 * 33 * sizeof(double) + align_up<float>(sizeof(float) * P.K * P.K, 16) +
+    return 16 + 2 * 33 * sizeof(double) + align_up<float>(sizeof(float) * P.K * P.kp, 16) +
            align_up<float>(sizeof(float) * P.ns, 16) +
            2 * sizeof(float) * (size_t)(band_tiles * TILE + P.K - 1) * P.Wp;
 }
@@ -80,80 +82,71 @@ __global__ void __launch_bounds__(RT_THREADS) k_fwd_rays(const Prob<float>* __re
     if (threadIdx.x == 0) flags[blockIdx.x] = L.bad ? 2 : (active != 0);
 }
 
-// One 4x4 output tile: out[r][c] = sum_{a,b} t[a][b] in[r + a][c + b + SHF]
-// (t = the taps in shared memory), looping over pairs of tap rows: rows a..a+4 of
-// the window serve tap rows a (output rows 0..3) and a+1 (output rows 0..3
-// from window rows a+1..a+4).
+// One 4x4 output tile: out[r][c] = sum_{a,b} t[a][b] in[r + a][c + b + SHF], NR
+// tap rows at a time held in registers (t: shared, rows of KP taps, loaded four
+// at a time).  What it runs into is shared-memory bandwidth: per warp and pair
+// of tap rows, five window rows of 16-byte loads (140 cycles at K = 21) beside
+// 168 cycles of FMAs an SM sub-partition; one load per tap (42 more cycles) put
+// it over.  Three rows at a time share more of the window where the registers
+// allow it.  (8 x 4 outputs a thread need half the window loads, but 128
+// registers a thread spill or leave half the warps idle: 15.8k against 12.4k
+// clocks at 128 x 128 and K = 11 on two SMs.)  Each output adds its terms in the
+// order a, b.
+template <int K, int NR>
+__device__ __forceinline__ void conv4_rows(unsigned src_a, int Wp, unsigned tap_a, float (&acc)[TILE][TILE]) {
+    constexpr int SHF = xoff_of<float>((K - 1) / 2) - (K - 1) / 2, KP = (K + 3) & ~3;
+    constexpr int NVW = (TILE + K - 1 + SHF + 3) / 4 * 4;
+    float t[NR][KP];
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+#pragma unroll
+        for (int v = 0; v < KP; v += 4) lds_vec(tap_a + (unsigned)((i * KP + v) * sizeof(float)), t[i] + v);
+#pragma unroll
+    for (int rr = 0; rr < TILE + NR - 1; ++rr) {
+        float in[NVW];
+#pragma unroll
+        for (int v = 0; v < NVW; v += 4) lds_vec(src_a + (unsigned)((rr * Wp + v) * sizeof(float)), in + v);
+#pragma unroll
+        for (int b = 0; b < K; ++b)
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const int r = rr - i;
+                if (r >= 0 && r < TILE) {
+#pragma unroll
+                    for (int c = 0; c < TILE; ++c) acc[r][c] = fmaf(t[i][b], in[SHF + b + c], acc[r][c]);
+                }
+            }
+    }
+}
 template <int K>
-__device__ __forceinline__ void conv_tile_pairs(const float* __restrict__ Pb, int Wp, const float* pt, float (&out)[16]) {
-    constexpr int HK = (K - 1) / 2;
-    constexpr int SHF = xoff_of<float>(HK) - HK;
-    constexpr int W = TILE + K - 1 + SHF;
-    constexpr int NVW = (W + 3) / 4 * 4;
-    const unsigned src_a = smem_addr(Pb);
-    float acc[TILE][TILE];
+__device__ __forceinline__ void conv4(const float* Pb, int Wp, const float* taps, float (&acc)[TILE][TILE]) {
+    constexpr int KP = (K + 3) & ~3, NR = K <= 13 ? 3 : 2, REST = K % NR;
+    const unsigned src = smem_addr(Pb), tap = smem_addr(taps);
 #pragma unroll
     for (int r = 0; r < TILE; ++r)
 #pragma unroll
         for (int c = 0; c < TILE; ++c) acc[r][c] = 0.f;
 #pragma unroll 1
-    for (int a = 0; a + 1 < K; a += 2) {
-#pragma unroll
-        for (int rr = 0; rr <= TILE; ++rr) {
-            float in[NVW];
-#pragma unroll
-            for (int v = 0; v < NVW; v += 4) lds_vec(src_a + (unsigned)(((a + rr) * Wp + v) * sizeof(float)), in + v);
-#pragma unroll
-            for (int b = 0; b < K; ++b) {
-                if (rr < TILE) {
-                    const float t = pt[a * K + b];
-#pragma unroll
-                    for (int c = 0; c < TILE; ++c) acc[rr][c] = fmaf(t, in[SHF + b + c], acc[rr][c]);
-                }
-                if (rr >= 1) {
-                    const float t = pt[(a + 1) * K + b];
-#pragma unroll
-                    for (int c = 0; c < TILE; ++c) acc[rr - 1][c] = fmaf(t, in[SHF + b + c], acc[rr - 1][c]);
-                }
-            }
-        }
-    }
-    if constexpr (K % 2 == 1) {  // the last tap row alone
-        constexpr int a = K - 1;
-#pragma unroll
-        for (int rr = 0; rr < TILE; ++rr) {
-            float in[NVW];
-#pragma unroll
-            for (int v = 0; v < NVW; v += 4) lds_vec(src_a + (unsigned)(((a + rr) * Wp + v) * sizeof(float)), in + v);
-#pragma unroll
-            for (int b = 0; b < K; ++b) {
-                const float t = pt[a * K + b];
-#pragma unroll
-                for (int c = 0; c < TILE; ++c) acc[rr][c] = fmaf(t, in[SHF + b + c], acc[rr][c]);
-            }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < TILE; ++r)
-#pragma unroll
-        for (int c = 0; c < TILE; ++c) out[r * 4 + c] = acc[r][c];
+    for (int a = 0; a + NR <= K; a += NR) conv4_rows<K, NR>(src + 4u * a * Wp, Wp, tap + 4u * a * KP, acc);
+    if constexpr (REST > 0) conv4_rows<K, REST>(src + 4u * (K - REST) * Wp, Wp, tap + 4u * (K - REST) * KP, acc);
 }
 
 template <int K>
 __global__ void __launch_bounds__(FWD_THREADS, 1) k_forward_band(const __grid_constant__ FwdArgs FA) {
+    constexpr int KP = (K + 3) & ~3;
     extern __shared__ __align__(16) unsigned char smem[];
     const Prob<float>& P = FA.probs[0];
     const CandScratch<float>& cs = FA.cs;
     const Geo<float> g = geo_of(P, 0);  // (the ray count is not used)
     double* red = reinterpret_cast<double*>(smem + 16);
     float* taps = reinterpret_cast<float*>(smem + 16 + 2 * 33 * sizeof(double));
-    float* s_sh = taps + align_up<float>(K * K, 4);
+    float* s_sh = taps + K * KP;
     float* band = s_sh + align_up<float>(g.ns, 4);
     const int tid = threadIdx.x, bs = blockDim.x;
-    // taps of B: the flipped PSF, row-major K x K
-    for (int i = tid; i < K * K; i += bs) {
-        const int a = i / K, b = i - a * K;
-        taps[i] = P.psf[(K - 1 - a) * K + (K - 1 - b)];
+    // taps of B: the flipped PSF, rows padded to KP
+    for (int i = tid; i < K * KP; i += bs) {
+        const int a = i / KP, b = i - a * KP;
+        taps[i] = b < K ? P.psf[(K - 1 - a) * K + (K - 1 - b)] : 0.f;
     }
     const int BT = FA.band_tiles, BR = BT * TILE;
     const int tiles_y = g.ntiles / g.tiles_x;
@@ -243,19 +236,19 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) k_forward_band(const __grid_co
                     sw[rr] = ld4(cs.swp + pp);
                     dv[rr] = ld4(cs.dpad + pp);
                 }
-                float o16[16];
-                conv_tile_pairs<K>(cur + (ty_l * TILE) * g.Wp + tx * TILE, g.Wp, taps, o16);
+                float acc[TILE][TILE];
+                conv4<K>(cur + (ty_l * TILE) * g.Wp + tx * TILE, g.Wp, taps, acc);
                 float ct = 0.f;  // the tile's 16 terms in FP32, then one FP64 add
 #pragma unroll
                 for (int rr = 0; rr < TILE; ++rr) {
                     const int y = ty * TILE + rr;
 #pragma unroll
                     for (int cc = 0; cc < TILE; ++cc) {
-                        const float res = sw[rr].v[cc] * (dv[rr].v[cc] - o16[rr * 4 + cc]);
+                        const float res = sw[rr].v[cc] * (dv[rr].v[cc] - acc[rr][cc]);
                         ct = fmaf(res, res, ct);
                         const int x = tx * TILE + cc;
                         if (FA.model && y < g.ny && x < g.nx)
-                            FA.model[(long long)k * g.nx * g.ny + y * g.nx + x] = o16[rr * 4 + cc];
+                            FA.model[(long long)k * g.nx * g.ny + y * g.nx + x] = acc[rr][cc];
                     }
                 }
                 chi += (double)ct;
