@@ -7,7 +7,10 @@
 // item of a call is.  k_cgls keeps one item on one SM and these images in an
 // L2-resident slab, so its convolutions wait for L2 and a call ends with one
 // SM at work.  Here C CTAs (1, 2, 4 or 8 SMs) share one item:
-//   * the image is cut into C bands of whole tile rows; each CTA keeps its
+//   * only tiles that hold a mapped pixel are convolved: L p is zero and sqrt(W)
+//     too elsewhere, so B L p is weighted away there and u is not read (60% of
+//     the tiles of the 256 x 256 system are left, 27% of the uneven batch's);
+//   * the image's rows with such tiles are cut into C bands of whole tile rows; each CTA keeps its
 //     band of L p and of W B L p, with the K - 1 halo rows, in its own shared
 //     memory.  A value in a neighbour's halo is also stored there, through
 //     distributed shared memory, when it is made;
@@ -81,59 +84,11 @@ __device__ __forceinline__ void cl_copy16(unsigned dst, const float* src) {
 }
 __device__ __forceinline__ void cl_copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// One tile of CT_ROWS x 4 outputs: out[r][c] = sum_{a,b} t[a][b] in[r + a][c +
-// b + SHF], NR tap rows at a time held in registers (t: shared, rows of
-// KP taps).  Shared-memory bandwidth is what a tile of 4 x 4 runs into (per
-// pair of tap rows and warp, 5 window rows: at K = 21 182 cycles of loads
-// against 168 of FMAs an SM sub-partition); 8 x 4 outputs share the taps and
-// most of the window rows (294 against 336).  Each output adds its terms in
-// the order a, b, as conv_tile does.
-constexpr int CT_ROWS = 4;
-template <int K, int NR>
-__device__ __forceinline__ void conv8_rows(unsigned src_a, int Wp, unsigned tap_a, float (&acc)[CT_ROWS][TILE]) {
-    constexpr int SHF = xoff_of<float>((K - 1) / 2) - (K - 1) / 2, KP = (K + 3) & ~3;
-    constexpr int NVW = (TILE + K - 1 + SHF + 3) / 4 * 4;
-    float t[NR][KP];
-#pragma unroll
-    for (int i = 0; i < NR; ++i)
-#pragma unroll
-        for (int v = 0; v < KP; v += 4) lds_vec(tap_a + (unsigned)((i * KP + v) * sizeof(float)), t[i] + v);
-#pragma unroll
-    for (int rr = 0; rr < CT_ROWS + NR - 1; ++rr) {
-        float in[NVW];
-#pragma unroll
-        for (int v = 0; v < NVW; v += 4) lds_vec(src_a + (unsigned)((rr * Wp + v) * sizeof(float)), in + v);
-#pragma unroll
-        for (int b = 0; b < K; ++b)
-#pragma unroll
-            for (int i = 0; i < NR; ++i) {
-                const int r = rr - i;
-                if (r >= 0 && r < CT_ROWS) {
-#pragma unroll
-                    for (int c = 0; c < TILE; ++c) acc[r][c] = fmaf(t[i][b], in[SHF + b + c], acc[r][c]);
-                }
-            }
-    }
-}
-template <int K>
-__device__ __forceinline__ void conv8(const float* Pb, int Wp, const float* taps, float (&acc)[CT_ROWS][TILE]) {
-    constexpr int KP = (K + 3) & ~3, NR = K <= 13 ? 3 : 2, REST = K % NR;
-    const unsigned src = smem_addr(Pb), tap = smem_addr(taps);
-#pragma unroll
-    for (int r = 0; r < CT_ROWS; ++r)
-#pragma unroll
-        for (int c = 0; c < TILE; ++c) acc[r][c] = 0.f;
-#pragma unroll 1
-    for (int a = 0; a + NR <= K; a += NR)
-        conv8_rows<K, NR>(src + 4u * a * Wp, Wp, tap + 4u * a * KP, acc);
-    if constexpr (REST > 0) conv8_rows<K, REST>(src + 4u * (K - REST) * Wp, Wp, tap + 4u * (K - REST) * KP, acc);
-}
-
 // How one problem is cut over C CTAs of NT threads (host and device)
 struct ClusterCut {
     int C, nt;
     int bt;       // tile rows per band
-    int blen;     // floats of one band buffer (bt tile rows, in pairs, + K - 1 rows)
+    int blen;     // floats of one band buffer (bt tile rows + K - 1 rows)
     int cap;      // source rows per CTA at most
     int blen2;    // floats allocated for the band of W B L p, which stages the rays of L^T too (stage of them)
     int stage;
@@ -143,7 +98,7 @@ struct ClusterCut {
         C = c;
         bt = (P.tiles_y + C - 1) / C;
         nt = bt * P.tiles_x > NTHREADS ? 2 * NTHREADS : NTHREADS;
-        blen = ((bt + CT_ROWS / TILE - 1) / (CT_ROWS / TILE) * CT_ROWS + P.K - 1) * P.Wp;
+        blen = (bt * TILE + P.K - 1) * P.Wp;
         cap = C == 1 ? P.sy : (5 * P.sy + 4 * C - 1) / (4 * C) + 1;
         const int q = bt * TILE * P.tiles_x * TILE;
         zlen = q > 4 * (cap + 1) * P.sx ? q : 4 * (cap + 1) * P.sx;
@@ -173,12 +128,12 @@ struct ClusterCtl {
 // Constants of the current item, written by thread 0 and read from shared
 // memory where they are used: held in registers they spill, and the shared
 // memory leaves too little L1 for the spilled lines of 512 threads (measured:
-// each phase paid an L2 round trip or two, 95k against 57k clocks an
+// each phase paid an L2 round trip or two, 95k against 71k clocks an
 // iteration of the 128 x 128 system).  Shared arrays are byte offsets.
 struct ClusterItem {
     Geo<float> g;
-    unsigned PA, PB, Z, p, h, gv, mi, mb;
-    int row0, ty0, ty1, hop, R, nx4, units, bt, blen, hn, stage;
+    unsigned PA, PB, Z, p, h, gv, mi, mb, tl;
+    int row0, ty0, ty1, tyA, tyB, hop, R, nx4, tiles, act, bt, blen, hn, stage;
     int i0, i1, pr0, pr1, hr0, hr1, e0, e1, cell0, cell1, r0, r1;
     float lamT;
     int cstat;
@@ -203,7 +158,7 @@ __host__ __device__ inline size_t ClusterCut::bytes(const Prob<float>& P) const 
     o += align_up<float>(sizeof(float) * (u.cap + 4) * P.sx, 16);                 // p
     o += align_up<float>(sizeof(float) * (P.nreg / P.ns) * (u.cap + 2) * P.sx, 16);  // H p
     o += 2 * align_up<float>(sizeof(float) * u.cap * P.sx, 16);                   // g, M^-1
-    o += align_up<float>(sizeof(unsigned short) * u.bt * P.tiles_x, 16);          // mapped-pixel bits of the tiles
+    o += 2 * align_up<float>(sizeof(unsigned short) * u.bt * P.tiles_x, 16);      // mapped-pixel bits of the tiles, tile list
     return o;
 }
 // global work space of one cluster
@@ -228,7 +183,7 @@ __device__ inline void cluster_item_fill(ClusterItem& I, const Prob<float>& P, c
     I.gv = carve(sizeof(float) * u.cap * P.sx);
     I.mi = carve(sizeof(float) * u.cap * P.sx);
     I.mb = carve(sizeof(unsigned short) * u.bt * P.tiles_x);
-    I.bt = u.bt;
+    I.tl = carve(sizeof(unsigned short) * u.bt * P.tiles_x);
     I.stage = u.stage;
     I.blen = u.blen;
     I.hn = (u.cap + 2) * P.sx;
@@ -257,16 +212,20 @@ __device__ inline void cluster_item_fill(ClusterItem& I, const Prob<float>& P, c
     I.cstat = cs.cstat[c];
     I.lam = A.lambdas[(long long)c * A.max_lam + k];
     I.lamT = (float)I.lam;
-    I.ty0 = min(rank * u.bt, P.tiles_y);
-    I.ty1 = min(I.ty0 + u.bt, P.tiles_y);
-    I.row0 = I.ty0 * TILE;
-    I.R = u.bt * TILE;
-    I.hop = I.R * P.Wp;  // from a band to the next
     I.nx4 = P.tiles_x * TILE;
-    I.units = (I.ty1 - I.ty0 + CT_ROWS / TILE - 1) / (CT_ROWS / TILE) * P.tiles_x;  // convolution tiles of CT_ROWS x 4
+    I.tyA = P.tiles_y;  // (the mapped tile rows follow)
+    I.tyB = 0;
 }
-// ... and, once the source rows are cut
-__device__ inline void cluster_item_rows(ClusterItem& I, const int* row, int rank) {
+// ... and, once the mapped tile rows [tyA, tyB) are known and the source rows cut
+__device__ inline void cluster_item_rows(ClusterItem& I, const int* row, int C, int rank) {
+    // bands of equal height; a halo reaches the next band only
+    I.bt = max((I.tyB - I.tyA + C - 1) / C, C > 1 ? (I.g.hk + TILE - 1) / TILE : 1);
+    I.ty0 = min(I.tyA + rank * I.bt, I.tyB);
+    I.ty1 = min(I.ty0 + I.bt, I.tyB);
+    I.row0 = I.ty0 * TILE;
+    I.R = I.bt * TILE;
+    I.hop = I.R * I.g.Wp;  // from a band to the next
+    I.tiles = (I.ty1 - I.ty0) * I.g.tiles_x;
     const int b0 = row[rank], b1 = row[rank + 1], sx = I.g.sx, sy = I.g.sy, ncx = I.g.ncx;
     I.i0 = b0 * sx;
     I.i1 = b1 * sx;
@@ -288,7 +247,7 @@ __device__ inline void cluster_item_rows(ClusterItem& I, const int* row, int ran
 // into Rs, sqrt(W) times it into Pb; mode 1: the convolution into Pc.
 template <int K, int NT>
 __device__ __noinline__ void cl_conv64(const ClusterItem& I, const double* src, float* hi, float* lo, const float* taps,
-                                       int mode) {
+                                       const unsigned short* tiles, int mode) {
     const Geo<float>& g = I.g;
     const int blen = I.blen, Wp = g.Wp, tiles_x = g.tiles_x, g0 = I.row0 * Wp;  // padded position of local position 0
     {
@@ -299,9 +258,10 @@ __device__ __noinline__ void cl_conv64(const ClusterItem& I, const double* src, 
         }
     }
     __syncthreads();
-    const int units = (I.ty1 - I.ty0) * TILE * tiles_x;  // four pixels of one row each
-    for (int t = threadIdx.x; t < units; t += NT) {
-        const int y = t / tiles_x, tx = t - y * tiles_x;
+    const unsigned short* list = tiles;
+    const int act = I.act, units = act * TILE;  // four pixels of one row each
+    for (int u = threadIdx.x; u < units; u += NT) {
+        const int r = u / act, t = list[u - r * act], ty = t / tiles_x, y = ty * TILE + r, tx = t - ty * tiles_x;
         const int base = y * Wp + tx * TILE + g.sh;
         float s[TILE], c[TILE];
 #pragma unroll
@@ -357,6 +317,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
     const Geo<float>& g = I.g;
     float* taps = reinterpret_cast<float*>(smem + CL_TAPS);
     auto sh = [&](unsigned o) { return reinterpret_cast<float*>(smem + o); };
+    auto tile_list = [&]() { return reinterpret_cast<const unsigned short*>(smem + I.tl); };
     ChainPos& ch = ctl->ch;  // (thread 0 of each CTA moves it)
     int fslot = 0, dslot = 0;  // halves of the warp-sum slots, alternated
 
@@ -476,14 +437,32 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
             }
             ctl->row[tid] = tid == 0 ? 0 : lo;
         }
+        {  // first and last tile row with a mapped pixel
+            int lo = I.g.plen, hi = 0;
+            const Entry<float>* E = I.E;
+            const int n = g.nent;
+#pragma unroll 8
+            for (int e = tid; e < n; e += NT) {
+                const int pp = E[e].ppos;
+                lo = min(lo, pp);
+                hi = max(hi, pp);
+            }
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0) {
+                atomicMin(&I.tyA, (lo / g.Wp - HK) / TILE);
+                atomicMax(&I.tyB, (hi / g.Wp - HK) / TILE + 1);
+            }
+        }
         __syncthreads();
         if (tid == 0) {
             const int cap = ClusterCut(A.probs[A.cand_prob[ch.c]], (int)C, A.max_smem).cap;
             ctl->row[C] = g.sy;
             for (int j = 1; j < (int)C; ++j)
                 ctl->row[j] = max(min(ctl->row[j], ctl->row[j - 1] + cap), max(ctl->row[j - 1], g.sy - ((int)C - j) * cap));
-            cluster_item_rows(I, ctl->row, (int)rank);
+            cluster_item_rows(I, ctl->row, (int)C, (int)rank);
         }
+        __syncthreads();
         for (int i = tid; i < 2 * K * KP; i += NT) {
             const int h = i / (K * KP), m = i - h * K * KP, a = m / KP, b = m - a * KP;
             // [0] flipped PSF (B), [1] PSF (B^T); rows padded to KP
@@ -501,6 +480,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
             for (int i = rank * part + tid; i < i1; i += NT) {
                 I.Pa[i] = 0.0;
                 I.Pb[i] = 0.0;
+                I.Rs[i] = 0.0;
             }
         }
         cl_sync();  // (a slice may lie in another CTA's band)
@@ -524,9 +504,9 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
         // ---- the own rays, with the owner of their pixel and its place there
         for (int e = I.e0 + tid; e < I.e1; e += NT) {
             const Entry<float> en = I.E[e];
-            const int R = I.R, y = en.ppos / g.Wp - HK, o = y / R, yl = y - o * R;
+            const int R = I.R, y = en.ppos / g.Wp - HK - I.tyA * TILE, o = y / R, yl = y - o * R;
             int4 q;
-            q.x = (en.ppos - o * I.hop) | (o << 20) | (o > 0 && yl < HK ? 1 << 24 : 0) |
+            q.x = (en.ppos - I.tyA * TILE * g.Wp - o * I.hop) | (o << 20) | (o > 0 && yl < HK ? 1 << 24 : 0) |
                   (o + 1 < (int)C && yl >= R - HK ? 1 << 25 : 0);
             q.y = en.base;
             q.z = __float_as_int(en.u);
@@ -544,13 +524,29 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
             cl_st(cl_map(smem_addr(smem) + I.PA + 4u * (m & 0xfffff), (m >> 20) & 15), 1.f);
         }
         cl_sync();
-        for (int t = tid; t < (I.ty1 - I.ty0) * g.tiles_x; t += NT) {
+        for (int t = tid; t < I.tiles; t += NT) {
             int ty, tx;
             tile_at(t, ty, tx);
             unsigned m = 0;
             for (int q = 0; q < 16; ++q)
                 if (sh(I.PA)[(ty * TILE + (q >> 2) + HK) * g.Wp + tx * TILE + (q & 3) + g.xoff] != 0.f) m |= 1u << q;
             reinterpret_cast<unsigned short*>(smem + I.mb)[t] = (unsigned short)m;
+        }
+        __syncthreads();
+        if (warp == 0) {  // the tiles to convolve, then the others
+            const unsigned short* mb = reinterpret_cast<const unsigned short*>(smem + I.mb);
+            unsigned short* list = reinterpret_cast<unsigned short*>(smem + I.tl);
+            int na = 0, nz = 0;
+            for (int t0 = 0; t0 < I.tiles; t0 += 32) {
+                const int t = t0 + lane;
+                const bool in = t < I.tiles, a = in && mb[t] != 0;
+                const unsigned am = __ballot_sync(0xffffffffu, a), zm = __ballot_sync(0xffffffffu, in && !a), below = (1u << lane) - 1u;
+                if (a) list[na + __popc(am & below)] = (unsigned short)t;
+                if (in && !a) list[I.tiles - 1 - nz - __popc(zm & below)] = (unsigned short)t;
+                na += __popc(am);
+                nz += __popc(zm);
+            }
+            if (lane == 0) I.act = na;
         }
         for (int t = tid; t < (I.ty1 - I.ty0) * TILE * I.nx4; t += NT) {  // Pa back to zero
             const int y = t / I.nx4, x = t - y * I.nx4;
@@ -573,7 +569,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
             while (run0 < I.r1 - I.r0 && I.rec[I.r0 + run0].y == I.rec[I.r0 + run0 - 1].y) ++run0;
 
         // ---- ||rhs|| = ||L^T B^T W d|| in FP64
-        cl_conv64<K, NT>(I, I.Pb, sh(I.PA), sh(I.PB), taps + K * KP, 1);
+        cl_conv64<K, NT>(I, I.Pb, sh(I.PA), sh(I.PB), taps + K * KP, tile_list(), 1);
         cl_sync();
         for (int i = I.i0 + tid; i < I.i1; i += NT) {
             const int ib = i / g.sx, ia = i - ib * g.sx;
@@ -607,7 +603,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 if (g.nreg > g.ns) I.h64[g.ns + i] = apply_H_row<float, double>(g, I.x64, g.ns + i);
             }
             cl_sync();
-            cl_conv64<K, NT>(I, I.Pa, sh(I.PA), sh(I.PB), taps, 0);
+            cl_conv64<K, NT>(I, I.Pa, sh(I.PA), sh(I.PB), taps, tile_list(), 0);
             cl_sync();
             dsum_start([&](int v) {
                 const int nt = g.ntiles, Wp = g.Wp;
@@ -615,6 +611,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 for (int t = v; t < nt; t += VT) {
                     int ty, tx;
                     tile_at(t, ty, tx);
+                    if (ty < I.tyA || ty >= I.tyB) continue;  // zeros
                     const double* q = I.Rs + (ty * TILE + HK) * Wp + tx * TILE + g.xoff;
                     double r[16];
 #pragma unroll
@@ -624,7 +621,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 }
                 return s;
             });
-            cl_conv64<K, NT>(I, I.Pb, sh(I.PA), sh(I.PB), taps + K * KP, 1);
+            cl_conv64<K, NT>(I, I.Pb, sh(I.PA), sh(I.PB), taps + K * KP, tile_list(), 1);
             cl_sync();
             if (rank == 0 && tid == 0) A.chi2[item_at()] = dsum_end();
             for (int i = I.i0 + tid; i < I.i1; i += NT) {
@@ -741,36 +738,44 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 cl_sync();  // bands of L p complete
                 // sqrt(W) B L p into Z, W B L p into the band and its neighbours' halos
                 {
-                    const int units = I.units, Wp = g.Wp, nx4 = I.nx4, xoff = g.xoff;
-                    for (int t = tid; t < units; t += NT) {
+                    const int act = I.act, Wp = g.Wp, nx4 = I.nx4, xoff = g.xoff;
+                    const unsigned short* list = tile_list();
+                    for (int i = I.tiles - 1 - tid; i >= act; i -= NT) {  // the others' zeros for delta's sum
                         int ty, tx;
-                        tile_at(t, ty, tx);
-                        const int y0 = ty * CT_ROWS, rows = min(CT_ROWS, (I.ty1 - I.ty0) * TILE - y0);
+                        tile_at(list[i], ty, tx);
+                        float* zt = sh(I.Z) + ty * TILE * nx4 + tx * TILE;
+#pragma unroll
+                        for (int r = 0; r < TILE; ++r) st4(zt + r * nx4, V4<float>{{0.f, 0.f, 0.f, 0.f}});
+                    }
+                    for (int i = tid; i < act; i += NT) {
+                        int ty, tx;
+                        tile_at(list[i], ty, tx);
+                        const int y0 = ty * TILE;
                         float* zt = sh(I.Z) + y0 * nx4 + tx * TILE;
                         // sqrt(W) of the tile arrives in its place of Z while it is convolved
                         const float* sg = I.swp + (I.row0 + y0 + HK) * Wp + tx * TILE + xoff;
-                        for (int r = 0; r < rows; ++r) cl_copy16(smem_addr(zt + r * nx4), sg + r * Wp);
-                        float acc[CT_ROWS][TILE];
-                        conv8<K>(sh(I.PA) + y0 * Wp + tx * TILE, Wp, taps, acc);
+#pragma unroll
+                        for (int r = 0; r < TILE; ++r) cl_copy16(smem_addr(zt + r * nx4), sg + r * Wp);
+                        float acc[TILE][TILE];
+                        conv4<K>(sh(I.PA) + y0 * Wp + tx * TILE, Wp, taps, acc);
                         cl_copy_wait();
                         const int R = I.R, hop = I.hop;
                         float* PB = sh(I.PB);
 #pragma unroll
-                        for (int r = 0; r < CT_ROWS; ++r)
-                            if (r < rows) {
-                                const int y = y0 + r, lp = (y + HK) * Wp + tx * TILE + xoff;
-                                const V4<float> sw = ld4(zt + r * nx4);
-                                V4<float> o, w;
+                        for (int r = 0; r < TILE; ++r) {
+                            const int y = y0 + r, lp = (y + HK) * Wp + tx * TILE + xoff;
+                            const V4<float> sw = ld4(zt + r * nx4);
+                            V4<float> o, w;
 #pragma unroll
-                                for (int cc = 0; cc < 4; ++cc) {
-                                    o.v[cc] = sw.v[cc] * acc[r][cc];
-                                    w.v[cc] = sw.v[cc] * o.v[cc];
-                                }
-                                st4(zt + r * nx4, o);
-                                st4(PB + lp, w);
-                                if (rank > 0 && y < HK) cl_st4(cl_map(smem_addr(PB + lp + hop), rank - 1), w.v);
-                                if (rank + 1 < C && y >= R - HK) cl_st4(cl_map(smem_addr(PB + lp) - 4u * hop, rank + 1), w.v);
+                            for (int cc = 0; cc < 4; ++cc) {
+                                o.v[cc] = sw.v[cc] * acc[r][cc];
+                                w.v[cc] = sw.v[cc] * o.v[cc];
                             }
+                            st4(zt + r * nx4, o);
+                            st4(PB + lp, w);
+                            if (rank > 0 && y < HK) cl_st4(cl_map(smem_addr(PB + lp + hop), rank - 1), w.v);
+                            if (rank + 1 < C && y >= R - HK) cl_st4(cl_map(smem_addr(PB + lp) - 4u * hop, rank + 1), w.v);
+                        }
                     }
                 }
                 cl_sync();  // bands of W B L p and all of Z complete
@@ -780,18 +785,21 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                     const int nr = g.nreg, nt = g.ntiles, nx4 = I.nx4, bt = I.bt;
                     const unsigned Zs = smem_addr(smem) + I.Z;
                     float dh = 0.f, cq = 0.f, q[2][16];
+                    // (tiles outside the bands are zeros)
+                    const int tA = I.tyA * g.tiles_x, tB = min(I.tyB * g.tiles_x, nt), tyA = I.tyA;
+                    const int t0 = v + (tA > v ? (tA - v + VT - 1) / VT * VT : 0);
                     auto load_tiles = [&](int t) {
 #pragma unroll
                         for (int j = 0; j < 2; ++j) {
                             int ty, tx;
-                            tile_at(min(t + j * VT, nt - 1), ty, tx);
-                            const int o = ty / bt;
-                            const unsigned a = cl_map(Zs + 4u * ((ty - o * bt) * TILE * nx4 + tx * TILE), o);
+                            tile_at(min(t + j * VT, tB - 1), ty, tx);
+                            const int o = (ty - tyA) / bt;
+                            const unsigned a = cl_map(Zs + 4u * ((ty - tyA - o * bt) * TILE * nx4 + tx * TILE), o);
 #pragma unroll
                             for (int r = 0; r < TILE; ++r) cl_ld4(a + 4u * r * nx4, q[j] + 4 * r);
                         }
                     };
-                    load_tiles(v);
+                    load_tiles(t0);
                     for (int i = v; i < nr; i += 16 * VT) {
                         float h[16];
 #pragma unroll
@@ -799,39 +807,34 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
 #pragma unroll
                         for (int j = 0; j < 16; ++j) dh = fmaf(h[j], h[j], dh);
                     }
-                    for (int t = v; t < nt; t += 2 * VT) {
+                    for (int t = t0; t < tB; t += 2 * VT) {
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
-                            if (t + j * VT < nt) {
+                            if (t + j * VT < tB) {
 #pragma unroll
                                 for (int m = 0; m < 16; ++m) cq = fmaf(q[j][m], q[j][m], cq);
                             }
-                        if (t + 2 * VT < nt) load_tiles(t + 2 * VT);
+                        if (t + 2 * VT < tB) load_tiles(t + 2 * VT);
                     }
                     return fmaf(I.lamT, dh, cq);
                 });
                 // u = B^T W B L p of the own band, at mapped pixels (the others stay zero)
                 {
-                    const int units = I.units, Wp = g.Wp;
-                    for (int t = tid; t < units; t += NT) {
+                    const int act = I.act, Wp = g.Wp;
+                    const unsigned short* list = tile_list();
+                    for (int i = tid; i < act; i += NT) {
+                        const int t = list[i];
                         int ty, tx;
                         tile_at(t, ty, tx);
-                        float acc[CT_ROWS][TILE];
-                        conv8<K>(sh(I.PB) + ty * CT_ROWS * Wp + tx * TILE, Wp, taps + K * KP, acc);
-                        float* PA = sh(I.PA) + (ty * CT_ROWS + HK) * Wp + tx * TILE + g.xoff;
+                        float acc[TILE][TILE];
+                        conv4<K>(sh(I.PB) + ty * TILE * Wp + tx * TILE, Wp, taps + K * KP, acc);
+                        float* PA = sh(I.PA) + (ty * TILE + HK) * Wp + tx * TILE + g.xoff;
+                        const unsigned m = reinterpret_cast<unsigned short*>(smem + I.mb)[t];
 #pragma unroll
-                        for (int h = 0; h < CT_ROWS / TILE; ++h)
-                            if (CT_ROWS / TILE * ty + h < I.ty1 - I.ty0) {
-                                const unsigned m =
-                                    reinterpret_cast<unsigned short*>(smem + I.mb)[(CT_ROWS / TILE * ty + h) * g.tiles_x + tx];
+                        for (int r = 0; r < TILE; ++r)
 #pragma unroll
-                                for (int r = 0; r < TILE; ++r) {
-                                    float* dst = PA + (h * TILE + r) * Wp;
-#pragma unroll
-                                    for (int cc = 0; cc < 4; ++cc)
-                                        if (m & (1u << (r * 4 + cc))) dst[cc] = acc[h * TILE + r][cc];
-                                }
-                            }
+                            for (int cc = 0; cc < 4; ++cc)
+                                if (m & (1u << (r * 4 + cc))) PA[r * Wp + cc] = acc[r][cc];
                     }
                 }
                 cl_sync();  // u complete, delta's warp sums here, Z read
