@@ -59,6 +59,7 @@ const KernelTable& table() {
         fill_f32_gen(k);
         fill_f64(k);
         fill_fast(k);
+        fill_fast1(k);
         fill_iter(k);
         fill_fwd_band(k);
         fill_cluster_a(k);
@@ -336,12 +337,12 @@ const void* pick_fwd(int prec, int K) {
 
 // two-CTA-per-SM kernel when the problem qualifies (FP32 contexts only)
 template <typename T>
-const void* pick_fast(mirage_ctx* ctx, const Prob<T>& P, int mode) {
+const void* pick_fast(mirage_ctx* ctx, const Prob<T>& P, int mode, bool alone) {
     if (sizeof(T) != 4 || P.interp == MIRAGE_INTERP_BICUBIC) return nullptr;  // four-corner rays only
     const Prob<float>& Pf = *reinterpret_cast<const Prob<float>*>(&P);
     const size_t b = fast_smem_bytes(Pf);
     if (b == 0 || (long long)b > ctx->max_smem_sm / 2 - 1024 || Pf.K >= MAX_K) return nullptr;
-    return table().fast[Pf.K][0][mode];
+    return table().fast[Pf.K][alone][mode];  // (alone: one CTA per SM)
 }
 
 // The cluster kernel's choice for one problem (C = 0: not eligible).
@@ -785,6 +786,10 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     int n_used = 0;
     for (int p = 0; p < n_probs; ++p) n_used += cands_of[p] > 0;
     const int want = o.variant;
+    long long n_items = 0;
+    for (int c = 0; c < n_cand; ++c) n_items += n_lam[c];
+    // no more items than SMs (or one candidate at a time): each CTA has an SM
+    const bool alone = n_items <= ctx->sm_count || o.mode == MIRAGE_MODE_PLAIN;
     auto choose = [&](const Prob<T>& P, int& mode, bool& fast) -> const void* {
         fast = false;
         mode = 0;
@@ -796,14 +801,14 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         if (want == 3) m = 2;
         if (want == 7) m = 3;
         if (m > 0 && (n_used > 1 || P.K * P.K > MAX_PTAP)) m = 0;
-        const void* f = pick_fast<T>(ctx, P, m);
+        const void* f = pick_fast<T>(ctx, P, m, alone);
         if (!f && m == 1 && want == 0) {  // FFMA parameter taps are compiled for K = 9 only
             m = 2;
-            f = pick_fast<T>(ctx, P, 2);
+            f = pick_fast<T>(ctx, P, 2, alone);
         }
         if (!f && m > 0) {
             m = 0;
-            f = pick_fast<T>(ctx, P, 0);
+            f = pick_fast<T>(ctx, P, 0, alone);
         }
         if (f) {
             fast = true;
@@ -873,8 +878,6 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         }
         chain_budget = tw / (double)cgls_slots(ctx, 2);
     }
-    long long n_items = 0;
-    for (int c = 0; c < n_cand; ++c) n_items += n_lam[c];
     for (int c = 0; c < n_cand; ++c) {
         const Prob<T>& P = hp[prob_idx[c]];
         int place = pick_place<T>(ctx, P, o.place);

@@ -19,8 +19,8 @@ struct KernelTable {
     const void* rt_rays[2];   // two-launch ray trace: trace (many CTAs per candidate)
     const void* rt_cells[2];  //                       place (one CTA per candidate)
     const void* finalize[2];
-    // fast[K][v][mode]: two-CTA-per-SM FP32 kernel, v = 0 for ns <= 1024,
-    // 1 for ns <= 2304; mode = tap source (0 shared, 1 params FFMA, 2 params
+    // fast[K][v][mode]: two-CTA-per-SM FP32 kernel (ns <= 1024), v = 1 compiled
+    // for one CTA per SM; mode = tap source (0 shared, 1 params FFMA, 2 params
     // FFMA2, 3 params FFMA with TF32-rounded factors)
     const void* fast[MAX_K][2][4];
     // iter[prec][K]: fixed-iteration CGLS with the iteration L-curve
@@ -43,6 +43,7 @@ void fill_f32_k21(KernelTable& t);
 void fill_f32_gen(KernelTable& t);
 void fill_f64(KernelTable& t);
 void fill_fast(KernelTable& t);
+void fill_fast1(KernelTable& t);
 void fill_iter(KernelTable& t);
 void fill_fwd_band(KernelTable& t);
 void fill_cluster_a(KernelTable& t);
