@@ -10,10 +10,10 @@
 //   * only tiles that hold a mapped pixel are convolved: L p is zero and sqrt(W)
 //     too elsewhere, so B L p is weighted away there and u is not read (60% of
 //     the tiles of the 256 x 256 system are left, 27% of the uneven batch's);
-//   * the image's rows with such tiles are cut into C bands of whole tile rows; each CTA keeps its
-//     band of L p and of W B L p, with the K - 1 halo rows, in its own shared
-//     memory.  A value in a neighbour's halo is also stored there, through
-//     distributed shared memory, when it is made;
+//   * the image's rows with such tiles are cut into C bands of whole tile rows;
+//     each CTA keeps its band of L p and of W B L p, with the K - 1 halo rows,
+//     in its own shared memory.  A value in a neighbour's halo is also stored
+//     there, through distributed shared memory, when it is made;
 //   * the source rows are cut into C runs of about equal ray counts.  A CTA
 //     interpolates the rays of its own cells (L p, stored to the bands that
 //     hold the pixels), sums L^T over its own cells and one more cell row, so
@@ -22,9 +22,11 @@
 //   * every sum over the image or the source is added up as k_cgls adds it:
 //     its 256 threads own the tiles and source pixels t = v + 256 k, so the
 //     terms are stored and virtual thread v's terms are added in that order,
-//     the last warps of each CTA taking one warp of virtual threads each.  An item's results are thus
-//     bit for bit those of k_cgls, for any C.
+//     the last warps of each CTA taking one warp of virtual threads each.  An
+//     item's results are thus bit for bit those of k_cgls, for any C.
 #pragma once
+
+#include <type_traits>
 
 #include "forward.cuh"
 
@@ -317,6 +319,17 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
     const Geo<float>& g = I.g;
     float* taps = reinterpret_cast<float*>(smem + CL_TAPS);
     auto sh = [&](unsigned o) { return reinterpret_cast<float*>(smem + o); };
+    // tiles by rows where there are fewer tiles than threads: a whole tile, two
+    // rows or one row a thread (a warp alone on its scheduler takes as long for
+    // 92 tiles as for 512)
+    auto by_rows = [&](int act, auto&& f) {
+        if (2 * act > NT)
+            f(std::integral_constant<int, 4>());
+        else if (4 * act > NT)
+            f(std::integral_constant<int, 2>());
+        else
+            f(std::integral_constant<int, 1>());
+    };
     auto tile_list = [&]() { return reinterpret_cast<const unsigned short*>(smem + I.tl); };
     ChainPos& ch = ctl->ch;  // (thread 0 of each CTA moves it)
     int fslot = 0, dslot = 0;  // halves of the warp-sum slots, alternated
@@ -747,36 +760,40 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
 #pragma unroll
                         for (int r = 0; r < TILE; ++r) st4(zt + r * nx4, V4<float>{{0.f, 0.f, 0.f, 0.f}});
                     }
-                    for (int i = tid; i < act; i += NT) {
-                        int ty, tx;
-                        tile_at(list[i], ty, tx);
-                        const int y0 = ty * TILE;
-                        float* zt = sh(I.Z) + y0 * nx4 + tx * TILE;
-                        // sqrt(W) of the tile arrives in its place of Z while it is convolved
-                        const float* sg = I.swp + (I.row0 + y0 + HK) * Wp + tx * TILE + xoff;
+                    const int R = I.R, hop = I.hop;
+                    by_rows(act, [&](auto rt) {
+                        constexpr int RT = decltype(rt)::value;
+                        for (int i = tid; i < act * (TILE / RT); i += NT) {
+                            const int part = i / act;
+                            int ty, tx;
+                            tile_at(list[i - part * act], ty, tx);
+                            const int y0 = ty * TILE + part * RT;
+                            float* zt = sh(I.Z) + y0 * nx4 + tx * TILE;
+                            // sqrt(W) of the rows arrives in its place of Z while they are convolved
+                            const float* sg = I.swp + (I.row0 + y0 + HK) * Wp + tx * TILE + xoff;
 #pragma unroll
-                        for (int r = 0; r < TILE; ++r) cl_copy16(smem_addr(zt + r * nx4), sg + r * Wp);
-                        float acc[TILE][TILE];
-                        conv4<K>(sh(I.PA) + y0 * Wp + tx * TILE, Wp, taps, acc);
-                        cl_copy_wait();
-                        const int R = I.R, hop = I.hop;
-                        float* PB = sh(I.PB);
+                            for (int r = 0; r < RT; ++r) cl_copy16(smem_addr(zt + r * nx4), sg + r * Wp);
+                            float acc[RT][TILE];
+                            conv4<K, RT>(sh(I.PA) + y0 * Wp + tx * TILE, Wp, taps, acc);
+                            cl_copy_wait();
+                            float* PB = sh(I.PB);
 #pragma unroll
-                        for (int r = 0; r < TILE; ++r) {
-                            const int y = y0 + r, lp = (y + HK) * Wp + tx * TILE + xoff;
-                            const V4<float> sw = ld4(zt + r * nx4);
-                            V4<float> o, w;
+                            for (int r = 0; r < RT; ++r) {
+                                const int y = y0 + r, lp = (y + HK) * Wp + tx * TILE + xoff;
+                                const V4<float> sw = ld4(zt + r * nx4);
+                                V4<float> o, w;
 #pragma unroll
-                            for (int cc = 0; cc < 4; ++cc) {
-                                o.v[cc] = sw.v[cc] * acc[r][cc];
-                                w.v[cc] = sw.v[cc] * o.v[cc];
+                                for (int cc = 0; cc < 4; ++cc) {
+                                    o.v[cc] = sw.v[cc] * acc[r][cc];
+                                    w.v[cc] = sw.v[cc] * o.v[cc];
+                                }
+                                st4(zt + r * nx4, o);
+                                st4(PB + lp, w);
+                                if (rank > 0 && y < HK) cl_st4(cl_map(smem_addr(PB + lp + hop), rank - 1), w.v);
+                                if (rank + 1 < C && y >= R - HK) cl_st4(cl_map(smem_addr(PB + lp) - 4u * hop, rank + 1), w.v);
                             }
-                            st4(zt + r * nx4, o);
-                            st4(PB + lp, w);
-                            if (rank > 0 && y < HK) cl_st4(cl_map(smem_addr(PB + lp + hop), rank - 1), w.v);
-                            if (rank + 1 < C && y >= R - HK) cl_st4(cl_map(smem_addr(PB + lp) - 4u * hop, rank + 1), w.v);
                         }
-                    }
+                    });
                 }
                 cl_sync();  // bands of W B L p and all of Z complete
                 // delta = p^T A p = ||sqrt(W) B L p||^2 + lam ||H p||^2
@@ -822,20 +839,24 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 {
                     const int act = I.act, Wp = g.Wp;
                     const unsigned short* list = tile_list();
-                    for (int i = tid; i < act; i += NT) {
-                        const int t = list[i];
-                        int ty, tx;
-                        tile_at(t, ty, tx);
-                        float acc[TILE][TILE];
-                        conv4<K>(sh(I.PB) + ty * TILE * Wp + tx * TILE, Wp, taps + K * KP, acc);
-                        float* PA = sh(I.PA) + (ty * TILE + HK) * Wp + tx * TILE + g.xoff;
-                        const unsigned m = reinterpret_cast<unsigned short*>(smem + I.mb)[t];
+                    by_rows(act, [&](auto rt) {
+                        constexpr int RT = decltype(rt)::value;
+                        for (int i = tid; i < act * (TILE / RT); i += NT) {
+                            const int part = i / act, t = list[i - part * act];
+                            int ty, tx;
+                            tile_at(t, ty, tx);
+                            const int y0 = ty * TILE + part * RT;
+                            float acc[RT][TILE];
+                            conv4<K, RT>(sh(I.PB) + y0 * Wp + tx * TILE, Wp, taps + K * KP, acc);
+                            float* PA = sh(I.PA) + (y0 + HK) * Wp + tx * TILE + g.xoff;
+                            const unsigned m = reinterpret_cast<unsigned short*>(smem + I.mb)[t] >> (4 * part * RT);
 #pragma unroll
-                        for (int r = 0; r < TILE; ++r)
+                            for (int r = 0; r < RT; ++r)
 #pragma unroll
-                            for (int cc = 0; cc < 4; ++cc)
-                                if (m & (1u << (r * 4 + cc))) PA[r * Wp + cc] = acc[r][cc];
-                    }
+                                for (int cc = 0; cc < 4; ++cc)
+                                    if (m & (1u << (r * 4 + cc))) PA[r * Wp + cc] = acc[r][cc];
+                        }
+                    });
                 }
                 cl_sync();  // u complete, delta's warp sums here, Z read
                 if (tid == 0) {
@@ -976,17 +997,28 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                     const double gnew = fsum_end();
                     const int it = ++ctl->it;
                     ++ctl->total_it;
-                    const double rel = sqrt(gnew / ctl->g0);
-                    if (!isfinite(gnew)) {
-                        ctl->brk = 1;
-                        ctl->stop = 1;
-                    } else if (!(rel > ctl->target) || ctl->total_it >= (A.maxit > 0 ? A.maxit : 25 * g.ns)) {
-                        ctl->stop = 1;
-                    } else if (rel < 0.5 * ctl->best) {
-                        ctl->best = rel;
-                        ctl->best_it = it;
-                    } else if (it - ctl->best_it > max(4000, 2 * g.ns)) {
-                        ctl->stop = 1;
+                    // The decisions of k_cgls, with rel = sqrt(gnew / g0): in FP64 only
+                    // where a single-precision ratio (good to 1e-6) leaves them open
+                    const float ratio = __fdividef((float)gnew, (float)ctl->g0);
+                    const float tt = (float)ctl->target, hb = 0.5f * (float)ctl->best;
+                    const bool clear = (float)gnew > 1e-30f && (float)ctl->g0 > 1e-30f && ratio < 1e30f &&
+                                       ratio > 1.0001f * (tt * tt) && ratio > 1.0001f * (hb * hb);
+                    if (clear && ctl->total_it < (A.maxit > 0 ? A.maxit : 25 * g.ns) &&
+                        it - ctl->best_it <= max(4000, 2 * g.ns)) {
+                        // above the target and no halving of the residual: go on
+                    } else {
+                        const double rel = sqrt(gnew / ctl->g0);
+                        if (!isfinite(gnew)) {
+                            ctl->brk = 1;
+                            ctl->stop = 1;
+                        } else if (!(rel > ctl->target) || ctl->total_it >= (A.maxit > 0 ? A.maxit : 25 * g.ns)) {
+                            ctl->stop = 1;
+                        } else if (rel < 0.5 * ctl->best) {
+                            ctl->best = rel;
+                            ctl->best_it = it;
+                        } else if (it - ctl->best_it > max(4000, 2 * g.ns)) {
+                            ctl->stop = 1;
+                        }
                     }
                 }
                 __syncthreads();

@@ -82,8 +82,8 @@ __global__ void __launch_bounds__(RT_THREADS) k_fwd_rays(const Prob<float>* __re
     if (threadIdx.x == 0) flags[blockIdx.x] = L.bad ? 2 : (active != 0);
 }
 
-// One 4x4 output tile: out[r][c] = sum_{a,b} t[a][b] in[r + a][c + b + SHF], NR
-// tap rows at a time held in registers (t: shared, rows of KP taps, loaded four
+// RT rows of a 4x4 output tile: out[r][c] = sum_{a,b} t[a][b] in[r + a][c + b +
+// SHF], NR tap rows at a time held in registers (t: shared, rows of KP taps, loaded four
 // at a time).  What it runs into is shared-memory bandwidth: per warp and pair
 // of tap rows, five window rows of 16-byte loads (140 cycles at K = 21) beside
 // 168 cycles of FMAs an SM sub-partition; one load per tap (42 more cycles) put
@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(RT_THREADS) k_fwd_rays(const Prob<float>* __re
 // registers a thread spill or leave half the warps idle: 15.8k against 12.4k
 // clocks at 128 x 128 and K = 11 on two SMs.)  Each output adds its terms in the
 // order a, b.
-template <int K, int NR>
-__device__ __forceinline__ void conv4_rows(unsigned src_a, int Wp, unsigned tap_a, float (&acc)[TILE][TILE]) {
+template <int K, int NR, int RT>
+__device__ __forceinline__ void conv4_rows(unsigned src_a, int Wp, unsigned tap_a, float (&acc)[RT][TILE]) {
     constexpr int SHF = xoff_of<float>((K - 1) / 2) - (K - 1) / 2, KP = (K + 3) & ~3;
     constexpr int NVW = (TILE + K - 1 + SHF + 3) / 4 * 4;
     float t[NR][KP];
@@ -102,7 +102,7 @@ __device__ __forceinline__ void conv4_rows(unsigned src_a, int Wp, unsigned tap_
 #pragma unroll
         for (int v = 0; v < KP; v += 4) lds_vec(tap_a + (unsigned)((i * KP + v) * sizeof(float)), t[i] + v);
 #pragma unroll
-    for (int rr = 0; rr < TILE + NR - 1; ++rr) {
+    for (int rr = 0; rr < RT + NR - 1; ++rr) {
         float in[NVW];
 #pragma unroll
         for (int v = 0; v < NVW; v += 4) lds_vec(src_a + (unsigned)((rr * Wp + v) * sizeof(float)), in + v);
@@ -111,24 +111,24 @@ __device__ __forceinline__ void conv4_rows(unsigned src_a, int Wp, unsigned tap_
 #pragma unroll
             for (int i = 0; i < NR; ++i) {
                 const int r = rr - i;
-                if (r >= 0 && r < TILE) {
+                if (r >= 0 && r < RT) {
 #pragma unroll
                     for (int c = 0; c < TILE; ++c) acc[r][c] = fmaf(t[i][b], in[SHF + b + c], acc[r][c]);
                 }
             }
     }
 }
-template <int K>
-__device__ __forceinline__ void conv4(const float* Pb, int Wp, const float* taps, float (&acc)[TILE][TILE]) {
+template <int K, int RT = TILE>
+__device__ __forceinline__ void conv4(const float* Pb, int Wp, const float* taps, float (&acc)[RT][TILE]) {
     constexpr int KP = (K + 3) & ~3, NR = K <= 13 ? 3 : 2, REST = K % NR;
     const unsigned src = smem_addr(Pb), tap = smem_addr(taps);
 #pragma unroll
-    for (int r = 0; r < TILE; ++r)
+    for (int r = 0; r < RT; ++r)
 #pragma unroll
         for (int c = 0; c < TILE; ++c) acc[r][c] = 0.f;
 #pragma unroll 1
-    for (int a = 0; a + NR <= K; a += NR) conv4_rows<K, NR>(src + 4u * a * Wp, Wp, tap + 4u * a * KP, acc);
-    if constexpr (REST > 0) conv4_rows<K, REST>(src + 4u * (K - REST) * Wp, Wp, tap + 4u * (K - REST) * KP, acc);
+    for (int a = 0; a + NR <= K; a += NR) conv4_rows<K, NR, RT>(src + 4u * a * Wp, Wp, tap + 4u * a * KP, acc);
+    if constexpr (REST > 0) conv4_rows<K, REST, RT>(src + 4u * (K - REST) * Wp, Wp, tap + 4u * (K - REST) * KP, acc);
 }
 
 template <int K>
