@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
         // this thread's first ray of L^T, where one stage holds them all (see there)
         auto run_at = [](int t, int n) { return (int)((long long)t * n / NT); };
         int run0 = run_at(tid, I.r1 - I.r0);
-        if (tid > 0)
+        if (run0 > 0)  // (with fewer rays than threads several shares start at 0)
             while (run0 < I.r1 - I.r0 && I.rec[I.r0 + run0].y == I.rec[I.r0 + run0 - 1].y) ++run0;
 
         // ---- ||rhs|| = ||L^T B^T W d|| in FP64
@@ -909,7 +909,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                         const int k1 = run_at(tid + 1, n);
                         if (n < r1 - I.r0) {
                             k0 = run_at(tid, n);
-                            if (tid > 0)
+                            if (k0 > 0)
                                 while (k0 < n && __float_as_int(S[k0].w) == __float_as_int(S[k0 - 1].w)) ++k0;
                         }
                         if (k1 > k0) {

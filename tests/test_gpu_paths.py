@@ -90,3 +90,23 @@ def test_forward_every_compiled_psf(mods, ctx32, k, nx, ny, sub):
     assert int(st.item()) == 0
     assert np.abs(m_g.double().cpu().numpy() - m_o).max() <= 2e-6 * np.abs(m_o).max()
     np.testing.assert_allclose(c_g.cpu().numpy(), c_o, rtol=1e-4)
+
+
+@pytest.mark.parametrize("n", [1, 24])
+@pytest.mark.parametrize("nx,ny,sx,sy,k", [(32, 32, 16, 16, 13), (24, 20, 9, 24, 13), (28, 36, 24, 17, 15)])
+def test_cluster_few_rays(mods, nx, ny, sx, sy, k, n):
+    # fewer rays than threads in a CTA, and rays in the first source cell: a
+    # fresh context (its work space is zeros where the driver hands out zeros)
+    # and a used one against the general kernel (variant 4)
+    g = Geometry(nx, ny, 1.5 / max(nx, ny), sx, sy, -0.7, 0.7, -0.7, 0.7, k, 1, REG_LAPLACIAN)
+    prob = make_problem(g, seed=10, psf_sigma=2.0)
+    lens = np.tile(np.array([0.02, 0.8, 0.3, 0.0, 0.0, 0.0, 0.0]), (n, 1))
+    lams = synth.lambda_grid(2, 1e-2, 1.0)
+    ctx = mods.Context(0, mods.MIRAGE_FP32)
+    p = device_problem(prob)
+    run = lambda v: ctx.eval_batch([p], _lens_t(lens), [0] * n, _lam_t(lams, n), [2] * n, want_all_x=True, variant=v)
+    outs = [run(0), run(0), run(4), run(0)]
+    for key in KEYS:
+        for o in outs:
+            assert torch.equal(o[key], outs[2][key]), key
+    ctx.close()
