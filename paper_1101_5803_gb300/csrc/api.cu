@@ -134,7 +134,7 @@ struct mirage_ctx {
     std::map<const void*, int> smem_set;  // kernel -> dynamic smem attribute set
     std::map<std::pair<const void*, std::pair<int, size_t>>, int> cl_active;  // resident clusters of (kernel, size, smem)
     cudaStream_t cap_stream = nullptr;   // graphs are captured here and launched on the caller's stream
-    static constexpr int NSIDE = 16;
+    static constexpr int NSIDE = 32;
     cudaStream_t side[NSIDE] = {};  // concurrent kernel groups
     cudaEvent_t fork_ev = nullptr, join_ev[NSIDE] = {};
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // phase timing (opts.threads < 0)
@@ -354,11 +354,16 @@ struct ClusterPlan {
 };
 
 // Clocks of one CG iteration of problem P: `lat` as one item sees it, `thr`
-// the SM clocks that it takes up.  Fits to measured iterations (clocks / 1000):
-// the general kernel with everything in shared memory 45 at 64 x 64 and K = 15;
-// the cluster kernel 64 on two SMs and 39 on eight at 128 x 128 and K = 11, 144
-// on eight at 256 x 256 and K = 21, two CTAs of 256 threads 65 each on one SM at
-// 64 x 64 and K = 15.  The two-CTA kernel: 27.5 each of two at 64 x 64, K = 9.
+// the SM clocks that it takes up.  Fits to measured iterations, good to about
+// 20% (one candidate, one lambda, refinement included; clocks / 1000; image,
+// source, K: general kernel with everything in shared memory, then the cluster
+// kernel on 1, 2, 4 and 8 SMs):
+//   48 48 11: 43, 90, 55, 42, 33   48 32 15: 34, 47, 33, 25, 23
+//   64 32 15: 37, 55, 34, 28, 23   96 48 11: (96), 76, 48, 38, 30
+//   128 48 15: (172), -, 99, 78, 57   256 128 21: (1555), -, -, -, 159
+// (in brackets: not all in shared memory).  A source about as fine as the image
+// has its L^T summed ray by ray (`gather`), which costs both kernels clocks per
+// source pixel.  The two-CTA kernel: 27.5 each of two at 64 x 64, K = 9.
 struct IterCost {
     double lat, thr;
 };
@@ -368,18 +373,17 @@ IterCost fast_cost(const Prob<T>& P) {
     return {2.0 * c, c};
 }
 template <typename T>
-IterCost general_cost(const Prob<T>& P) {
-    const double c = 4.0 * P.K * P.K * P.npix / 100.0 + 2.0 * P.nrays;
+IterCost general_cost(const Prob<T>& P, bool in_smem) {
+    if (P.fft_m) return {6.0 * P.fft_m * P.fft_m, 6.0 * P.fft_m * P.fft_m};
+    const int per = (P.ntiles + NTHREADS - 1) / NTHREADS;
+    double c = 14500.0 + 73.0 * P.K * P.K * per + 1.5 * P.nrays + (4 * P.ncells > P.plen ? 7.2 * P.ns : 0.0);
+    if (!in_smem) c *= 1.6;
     return {c, c};
 }
 inline IterCost cluster_cost(const Prob<float>& P, int C, int nt) {
     const double conv = 4.0 * P.K * P.K * P.npix, rays = P.nrays;
-    if (C == 1) {
-        if (nt > NTHREADS) return {conv / 150.0 + 3.0 * rays + 16000.0, conv / 150.0 + 3.0 * rays + 16000.0};
-        return {conv / 90.0 + 5.0 * rays, conv / 180.0 + 2.5 * rays};
-    }
-    const double lat = (conv / 150.0 + 1.5 * rays) / C + 26000.0;
-    return {lat, lat * C * (nt > NTHREADS ? 1.0 : 0.7)};
+    const double lat = 20000.0 + 0.6 * rays + (conv / 170.0 + 3.5 * rays + (4 * P.ncells > P.plen ? 25.0 * P.ns : 0.0)) / C;
+    return {lat, lat * C * (nt > NTHREADS ? 1.0 : 0.85)};
 }
 
 // dynamic shared memory of a cluster-kernel CTA: two CTAs of 256 threads share
@@ -391,10 +395,8 @@ inline int cluster_smem_limit(const mirage_ctx* ctx, int nt) {
 template <typename T>
 bool cluster_fits(const mirage_ctx* ctx, const Prob<T>& P, int C, ClusterPlan& out) {
     if constexpr (sizeof(T) == 4) {
-        // one ray per pixel with four corners, the general kernel's per-cell
-        // form of L^T (its cell sums fit an image), a compiled PSF width
-        if (P.Np != 1 || P.interp == MIRAGE_INTERP_BICUBIC || P.fft_m || P.K >= MAX_K || 4 * P.ncells > P.plen ||
-            !table().cluster[P.K][0])
+        // one ray per pixel with four corners, a compiled PSF width
+        if (P.Np != 1 || P.interp == MIRAGE_INTERP_BICUBIC || P.fft_m || P.K >= MAX_K || !table().cluster[P.K][0])
             return false;
         const ClusterCut u(P, C, cluster_smem_limit(ctx, ClusterCut(P, C, 0).nt));
         // halos reach the next band only; ring positions have 20 bits
@@ -563,8 +565,8 @@ int launch_raytrace(mirage_ctx* ctx, const Prob<T>* dprobs, const int* dcand, co
     constexpr int prec = prec_of<T>();
     const KernelTable& tb = table();
     const size_t cells_smem = (size_t)max_cells * 4;
-    // Ray numbers in shared memory: two launches (measured, one 64 x 64 candidate:
-    // 30 us against 260 for one CTA; 256 candidates: 0.3 against 0.53 ms).  The
+    // Ray numbers in shared memory: two launches (one 64 x 64 candidate: 15 + 35 us;
+    // a whole forward call on it 282 -> 91 us against the trace on one CTA).  The
     // CTAs of the trace take at least RT_MIN_PIX pixels, and no more of them than
     // fill the device twice
     const size_t place_smem = sizeof(int) * (size_t)(max_cells + max_rays);
@@ -772,7 +774,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         int prob = -1;   // the single problem of the group, -2 if several
         int per_sm = 1;  // resident CTAs per SM
         long long slots = 0;  // CTAs (clusters) of the persistent launch
-        double cost = 0.0;     // estimated SM clocks of its items
+        double load = 0.0;     // estimated clocks of its items, one after another
         double longest = 0.0;  // estimated clocks of its longest item
         size_t smem = 0;
         long long slab = 0;
@@ -816,56 +818,78 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         }
         return f;
     };
-    // kernel of the problems that the two-CTA kernel does not take, unless a
-    // kernel or a placement of the general kernel is asked for: the general one
-    // where everything fits in shared memory, or the cluster kernel of one of its
-    // sizes, by the smallest estimated time: the problem's longest item, or the
-    // whole call's work on all SMs at that choice's efficiency.  (General against
-    // cluster kernel, measured: 64 candidates x 8 lambdas at 64 x 64 and K = 15
-    // 14.8 against 16.9 ms, one candidate 7.5 against 5.7 ms; 48 x 16 at 128 x 128,
-    // which does not fit, 277 against 210 ms)
-    std::vector<ClusterPlan> clp(n_probs);
-    std::vector<IterCost> cost_p(n_probs);
+    // Kernel of the items that the two-CTA kernel does not take, unless a kernel
+    // or a placement of the general kernel is asked for.  A problem has up to two
+    // forms: the one that takes the least SM time an iteration (the general kernel
+    // where everything fits in shared memory, or the cluster kernel of some size),
+    // and the one with the shortest iteration.  Items that would outlast the call
+    // in the first form take the second.  All forms give the same bits.  (48 x 48
+    // image and source, K = 15, one item: 23.7 us an iteration in the general
+    // kernel, 13.8 on a cluster of eight SMs; 304 such items 25 ms in the general
+    // kernel and 33 on clusters of four)
+    struct Form {
+        IterCost it;
+        ClusterPlan cp;  // C = 0: general kernel
+    };
+    std::vector<Form> cheap(n_probs), quick(n_probs);
+    double limit = 0.0;     // clocks that an item may take in its problem's cheap form
+    double call_time = 0.0;  // estimated clocks of the call
+    // form of an item of problem p with w iterations where items may take T_ clocks
+    auto form_of = [&](int p, double w, double T_) -> const Form& {
+        return w * cheap[p].it.lat > T_ && quick[p].it.lat < 0.8 * cheap[p].it.lat ? quick[p] : cheap[p];
+    };
     {
-        std::vector<std::vector<std::pair<IterCost, ClusterPlan>>> can(n_probs);
-        std::vector<double> weight(n_probs, 0.0), longest(n_probs, 0.0);
-        for (int c = 0; c < n_cand; ++c) {
-            for (int k = 0; k < n_lam[c]; ++k) weight[prob_idx[c]] += chain_weight(n_lam[c], k);
-            longest[prob_idx[c]] = std::max(longest[prob_idx[c]], chain_weight(n_lam[c], 0));
-        }
-        double total = 0.0;
+        std::map<std::pair<int, int>, int> classes;  // (problem, lambdas) -> candidates
+        for (int c = 0; c < n_cand; ++c) classes[{prob_idx[c], n_lam[c]}]++;
         for (int p = 0; p < n_probs; ++p) {
             if (!cands_of[p]) continue;
             int m = 0;
             bool f = false;
             const bool fast_p = choose(hp[p], m, f) != nullptr;
-            cost_p[p] = fast_p ? fast_cost(hp[p]) : general_cost(hp[p]);
+            cheap[p].it = fast_p ? fast_cost(hp[p]) : general_cost(hp[p], pick_place<T>(ctx, hp[p], o.place) == PLACE_SMEM);
+            quick[p] = cheap[p];
             if constexpr (sizeof(T) == 4) {
-                if (!fast_p && o.place == 0 && want != 4 && want != 5 && want != 6) {
-                    if (pick_place<T>(ctx, hp[p]) == PLACE_SMEM) can[p].push_back({general_cost(hp[p]), ClusterPlan()});
-                    for (int C = 1; C <= CL_MAX; C *= 2) {
-                        ClusterPlan cp;
-                        if (cluster_fits<T>(ctx, hp[p], C, cp)) can[p].push_back({cluster_cost(hp[p], C, cp.nt), cp});
-                    }
-                    double thr = can[p].empty() ? cost_p[p].thr : 1e300;
-                    for (auto& x : can[p]) thr = std::min(thr, x.first.thr);
-                    cost_p[p].thr = thr;
-                }
-            }
-            total += weight[p] * cost_p[p].thr;
-        }
-        for (int p = 0; p < n_probs; ++p) {
-            const double thr = cost_p[p].thr;
-            double best = 1e300;
-            for (auto& x : can[p]) {
-                const double est = std::max(longest[p] * x.first.lat, total / ctx->sm_count * x.first.thr / thr);
-                if (est < 0.95 * best) {
-                    best = est;
-                    clp[p] = x.second;
-                    cost_p[p] = x.first;
+                if (fast_p || o.place != 0 || want == 4 || want == 5 || want == 6) continue;
+                bool any = pick_place<T>(ctx, hp[p]) == PLACE_SMEM;
+                for (int C = 1; C <= CL_MAX; C *= 2) {
+                    Form x;
+                    if (!cluster_fits<T>(ctx, hp[p], C, x.cp)) continue;
+                    x.it = cluster_cost(hp[p], C, x.cp.nt);
+                    if (!any || x.it.thr < cheap[p].it.thr) cheap[p] = x;
+                    if (!any || x.it.lat < quick[p].it.lat) quick[p] = x;
+                    any = true;
                 }
             }
         }
+        // the call's time as a function of the limit: its longest item, or its work
+        // on all SMs, and part of the other one (the end of a call is never packed
+        // full)
+        bool two = false;
+        for (int p = 0; p < n_probs; ++p) two |= quick[p].it.lat < 0.8 * cheap[p].it.lat;
+        std::vector<std::vector<double>> w(max_lam + 1);
+        double total = 0.0, best = 1e300;
+        for (auto& x : classes) {
+            const int n = x.first.second;
+            for (int k = (int)w[n].size(); k < n; ++k) w[n].push_back(chain_weight(n, k));
+            for (int k = 0; k < n; ++k) total += x.second * w[n][k] * cheap[x.first.first].it.thr / ctx->sm_count;
+        }
+        for (double T_ = 0.5 * total; T_ < 1e3 * total; T_ *= 1.5) {
+            double sum = 0.0, longest = 0.0;
+            for (auto& x : classes)
+                for (double wk : w[x.first.second]) {
+                    const IterCost& it = form_of(x.first.first, wk, T_).it;
+                    sum += x.second * wk * it.thr / ctx->sm_count;
+                    longest = std::max(longest, wk * it.lat);
+                }
+            const double est = std::max(sum, longest) + 0.5 * std::min(sum, longest);
+            if (est < 0.98 * best) {
+                best = est;
+                limit = T_;
+                call_time = std::max(sum, longest);
+            }
+            if (!two || longest < T_) break;  // a larger limit changes nothing more
+        }
+        if (o.mode == MIRAGE_MODE_PLAIN) limit = 0.0;  // one candidate at a time
     }
     // chained calls: each CTA slot's share of the estimated cost of the call
     double chain_budget = 0.0;
@@ -900,29 +924,35 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
             item_slab = (long long)fast_slab_bytes(*reinterpret_cast<const Prob<float>*>(&P));
             per_sm = 2;
         }
-        const ClusterPlan& cp = clp[prob_idx[c]];
-        if (cp.C) {
-            fn = cp.fn;
-            item_smem = cp.smem;
-            item_slab = cp.slab;
-        }
-        if (!fn) {
+        // the group of candidate c's items of lambda k (chains: of the smallest lambda)
+        auto group_of = [&](int k) -> Group* {
+            const double w = chain_weight(n_lam[c], lam_start ? 0 : k);
+            const Form& form = form_of(prob_idx[c], w, limit);
+            const ClusterPlan& cp = form.cp;
+            const void* f = cp.C ? cp.fn : fn;
+            if (!f) return nullptr;
+            Group& g = groups[std::make_pair(f, cp.C ? 16 + cp.C : (int)big)];
+            g.fn = f;
+            g.big = big;
+            g.fast = fast;
+            g.cl = cp.C;
+            g.nt = cp.C ? cp.nt : NTHREADS;
+            g.prob = (g.prob == -1 || g.prob == prob_idx[c]) ? prob_idx[c] : -2;
+            g.per_sm = per_sm;
+            g.smem = std::max(g.smem, cp.C ? cp.smem : item_smem);
+            g.slab = std::max<long long>(g.slab, cp.C ? cp.slab : item_slab);
+            g.load += form.it.lat * chain_weight(n_lam[c], k);
+            g.longest = std::max(g.longest, form.it.lat * w);
+            return &g;
+        };
+        for (int k = n_lam[c] - 1; k > 0; --k)
+            if (lam_start) group_of(k);
+        Group* g0 = group_of(0);
+        if (!g0) {
             set_error("no kernel for this PSF size");
             return MIRAGE_ERR_UNSUPPORTED;
         }
-        auto key = std::make_pair(fn, cp.C ? 16 + cp.C : (int)big);
-        Group& g = groups[key];
-        g.fn = fn;
-        g.big = big;
-        g.fast = fast;
-        g.cl = cp.C;
-        g.nt = cp.C ? cp.nt : NTHREADS;
-        g.prob = (g.prob == -1 || g.prob == prob_idx[c]) ? prob_idx[c] : -2;
-        g.per_sm = per_sm;
-        g.smem = std::max(g.smem, item_smem);
-        g.slab = std::max<long long>(g.slab, item_slab);
-        for (int k = 0; k < n_lam[c]; ++k) g.cost += cost_p[prob_idx[c]].thr * chain_weight(n_lam[c], k);
-        g.longest = std::max(g.longest, cost_p[prob_idx[c]].lat * chain_weight(n_lam[c], 0));
+        Group& g = *g0;
         const double work = (double)P.plen * P.K * P.K + 8.0 * P.nrays;
         // lambda grids ascend: smaller k = smaller lambda = more CG iterations
         auto cost_of = [&](int k) { return work * (double)(n_lam[c] - k + 4); };
@@ -964,9 +994,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                 push_run(ka, n_lam[c] - 1, cd);
             }
         } else {
-            for (int k = 0; k < n_lam[c]; ++k) {
-                g.items.push_back({-cost_of(k), pack_chain(c, k, k)});
-            }
+            for (int k = 0; k < n_lam[c]; ++k) (k ? group_of(k) : g0)->items.push_back({-cost_of(k), pack_chain(c, k, k)});
         }
     }
     std::vector<int> all_items;
@@ -1188,21 +1216,20 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                 cudaEventRecord(ctx->fork_ev, st);
                 for (int i = 0; i < n_side; ++i) cudaStreamWaitEvent(ctx->side[i], ctx->fork_ev, 0);
             }
-            // Several groups share the device from the start, each with CTAs for
-            // its part of the estimated work, and each launches the rest of the CTAs
+            // Several groups share the device from the start, each with the CTAs that
+            // finish its items in the call's estimated time (and half as many more:
+            // iteration counts are estimates), and each launches the rest of the CTAs
             // that it could use behind them: those start as other groups end.  (One
             // group after the other, each on all SMs, leaves the last group's longest
-            // item alone on the device: the uneven batch of 48 candidates took 633 ms
-            // that way, 362 ms this way.)
-            double total_cost = 0.0;
-            for (Group* g : glist) total_cost += g->cost;
+            // item alone on the device: the uneven batch of 48 candidates then ran at
+            // 0.97 of the speed of the general kernels alone, side by side at 1.40.)
             for (int part = 0; part < (fork ? 2 : 1) && !rc; ++part)
                 for (size_t gi = 0; gi < glist.size() && !rc; ++gi) {
                     Group* g = glist[gi];
                     const cudaStream_t gs = fork ? ctx->side[(2 * gi + part) % ctx->NSIDE] : st;
                     const long long full = std::min<long long>(g->slots, (long long)g->items.size());
                     const long long first =
-                        fork ? std::min(full, std::max<long long>(1, (long long)std::llround(g->slots * g->cost / total_cost))) : full;
+                        fork ? std::min(full, std::max<long long>(1, (long long)std::ceil(1.5 * g->load / call_time))) : full;
                     const int grid = (int)(part == 0 ? first : full - first);
                     if (!grid) continue;
                     A.slab = ctx->slab.as<unsigned char>() + (g_slab_off[gi] + (part ? first : 0)) * slab_stride;
@@ -1266,7 +1293,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                     fn = ff;
                     item_smem = fast_smem_bytes(*reinterpret_cast<const Prob<float>*>(&P));
                 }
-                const ClusterPlan& cp = clp[prob_idx[c]];
+                const ClusterPlan& cp = form_of(prob_idx[c], 1.0, limit).cp;
                 if (cp.C) {
                     fn = cp.fn;
                     item_smem = cp.smem;

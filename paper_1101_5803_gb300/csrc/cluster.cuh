@@ -138,7 +138,7 @@ struct ClusterItem {
     int row0, ty0, ty1, tyA, tyB, hop, R, nx4, tiles, act, bt, blen, hn, stage;
     int i0, i1, pr0, pr1, hr0, hr1, e0, e1, cell0, cell1, r0, r1;
     float lamT;
-    int cstat;
+    int cstat, gather;
     double lam;
     double *Pa, *Pb, *Pc, *Rs, *x64, *xb, *sv, *h64;
     float *gvg, *zg, *xg, *hg;
@@ -215,6 +215,7 @@ __device__ inline void cluster_item_fill(ClusterItem& I, const Prob<float>& P, c
     I.lam = A.lambdas[(long long)c * A.max_lam + k];
     I.lamT = (float)I.lam;
     I.nx4 = P.tiles_x * TILE;
+    I.gather = 4 * P.ncells > P.plen;  // the form of L^T that k_cgls takes
     I.tyA = P.tiles_y;  // (the mapped tile rows follow)
     I.tyB = 0;
 }
@@ -329,6 +330,11 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
             f(std::integral_constant<int, 2>());
         else
             f(std::integral_constant<int, 1>());
+    };
+    auto clear_stage = [&]() {  // the staged rays of L^T
+        float* PB = sh(I.PB);
+        const int n = min(I.blen, 4 * min(I.stage, I.r1 - I.r0));
+        for (int i = tid; i < n; i += NT) PB[i] = 0.f;
     };
     auto tile_list = [&]() { return reinterpret_cast<const unsigned short*>(smem + I.tl); };
     ChainPos& ch = ctl->ch;  // (thread 0 of each CTA moves it)
@@ -874,7 +880,10 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 // equal run of whole cells (a cell belongs to the run that its first
                 // ray falls in), so that the lanes of a warp stay about equally busy:
                 // one cell a lane had a warp wait for its fullest cell (measured:
-                // 12k against 5k clocks at 128 x 128 on two SMs)
+                // 12k against 5k clocks at 128 x 128 on two SMs).
+                // Where the cell sums would not fit an image (a source about as fine as
+                // the image), k_cgls sums each source pixel's rays directly, and so does
+                // this: then the rays are only staged, with the starts of their cells
                 {
                     float4* S = reinterpret_cast<float4*>(sh(I.PB));
                     const float* PA = sh(I.PA);
@@ -882,9 +891,16 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                     const int4* rec = I.rec;
                     float4* Zc = reinterpret_cast<float4*>(sh(I.Z)) - I.hr0 * g.sx;  // indexed by the cell's base
                     const int n4 = I.i1 - I.hr0 * g.sx;
-                    for (int i = tid; i < n4; i += NT) Zc[I.hr0 * g.sx + i] = make_float4(0.f, 0.f, 0.f, 0.f);
                     const int r1 = I.r1, stage = I.stage;
+                    const bool gather = I.gather;
+                    if (gather) {
+                        int* cz = reinterpret_cast<int*>(sh(I.Z));
+                        for (int i = I.cell0 + tid; i <= I.cell1; i += NT) cz[i - I.cell0] = I.cst[i] - I.r0;
+                    } else {
+                        for (int i = tid; i < n4; i += NT) Zc[I.hr0 * g.sx + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
                     for (int s0 = I.r0; s0 < r1; s0 += stage) {
+                        if (gather && r1 - I.r0 > stage) break;  // (read where they are)
                         const int n = min(stage, r1 - s0);
                         for (int e = tid; e < n; e += 8 * NT) {
                             int4 q[8];
@@ -901,6 +917,7 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                                 if (e + j * NT < n)
                                     S[e + j * NT] = make_float4(U[j], __int_as_float(q[j].z), __int_as_float(q[j].w), __int_as_float(q[j].y));
                         }
+                        if (gather) break;
                         __syncthreads();
                         // this thread's run [k0, k1): from the first cell start at or after its
                         // share's start to the next thread's.  A cell that the stage cuts
@@ -948,15 +965,42 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                     const float a = ctl->a, lamT = I.lamT, invNp = g.invNp;
                     const int sx = g.sx, sy = g.sy, i0 = I.i0, i1 = I.i1;
                     const float* cp = sh(I.Z) - 4 * I.hr0 * sx;
+                    const bool gather = I.gather, staged = I.r1 - I.r0 <= I.stage;
+                    auto ray_at = [&](int k) {  // ray r0 + k: U, u, v
+                        if (staged) return reinterpret_cast<const float4*>(sh(I.PB))[k];
+                        const int4 q = I.rec[I.r0 + k];
+                        const unsigned o = (q.x >> 20) & 15;
+                        const float U = cl_ld(cl_map(smem_addr(smem) + I.PA + 4u * (q.x & 0xfffff), o));
+                        return make_float4(U, __int_as_float(q.z), __int_as_float(q.w), 0.f);
+                    };
                     const float* hx = sh(I.h) - I.hr0 * sx;
                     float *gv_sh = sh(I.gv) - i0, *mi = sh(I.mi) - i0;
                     for (int i = i0 + tid; i < i1; i += NT) {
                         const int ib = i / sx, ia = i - ib * sx;
                         float acc = 0.f;
-                        if (ib <= sy - 2 && ia <= sx - 2) acc += cp[4 * i + 0];
-                        if (ib <= sy - 2 && ia >= 1) acc += cp[4 * (i - 1) + 1];
-                        if (ib >= 1 && ia <= sx - 2) acc += cp[4 * (i - sx) + 2];
-                        if (ib >= 1 && ia >= 1) acc += cp[4 * (i - sx - 1) + 3];
+                        if (gather) {
+#pragma unroll
+                            for (int d = 0; d < 4; ++d) {
+                                const int iy0 = ib - (d >> 1), ix0 = ia - (d & 1);
+                                if (iy0 < 0 || iy0 > sy - 2 || ix0 < 0 || ix0 > sx - 2) continue;
+                                const int* cz = reinterpret_cast<const int*>(sh(I.Z)) + (iy0 * (sx - 1) + ix0 - I.cell0);
+                                const int k1 = cz[1];
+                                for (int k = cz[0]; k < k1; k += 4) {  // four rays' loads together
+                                    float4 r[4];
+#pragma unroll
+                                    for (int j = 0; j < 4; ++j) r[j] = ray_at(min(k + j, k1 - 1));
+#pragma unroll
+                                    for (int j = 0; j < 4; ++j)
+                                        if (k + j < k1)
+                                            acc = fmaf((d & 1 ? r[j].y : 1.f - r[j].y) * (d & 2 ? r[j].z : 1.f - r[j].z), r[j].x, acc);
+                                }
+                            }
+                        } else {
+                            if (ib <= sy - 2 && ia <= sx - 2) acc += cp[4 * i + 0];
+                            if (ib <= sy - 2 && ia >= 1) acc += cp[4 * (i - 1) + 1];
+                            if (ib >= 1 && ia <= sx - 2) acc += cp[4 * (i - sx) + 2];
+                            if (ib >= 1 && ia >= 1) acc += cp[4 * (i - sx - 1) + 3];
+                        }
                         float ht;
                         if (g.reg == 1) {
                             const float* hy = hx + I.hn;
@@ -966,17 +1010,16 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                         } else {
                             ht = apply_HT_at<float, float>(g, hx, i, ia, ib);
                         }
-                        const float ap = acc * invNp + lamT * ht;
+                        const float ap = gather ? fmaf(lamT, ht, acc) : acc * invNp + lamT * ht;  // (invNp = 1)
                         const float gv = fmaf(-a, ap, gv_sh[i]);
                         gv_sh[i] = gv;
                         I.gvg[i] = gv;
                         I.zg[i] = mi[i] * gv;
                     }
-                    float* PB = sh(I.PB);
-                    const int n = min(I.blen, 4 * min(I.stage, I.r1 - I.r0));
-                    for (int i = tid; i < n; i += NT) PB[i] = 0.f;  // the staged rays
+                    if (!gather) clear_stage();
                 }
                 cl_sync();  // g and z complete
+                if (I.gather) clear_stage();
                 fsum_start(grad_chain);
                 {
                     const float a = ctl->a;

@@ -92,6 +92,25 @@ def test_forward_every_compiled_psf(mods, ctx32, k, nx, ny, sub):
     np.testing.assert_allclose(c_g.cpu().numpy(), c_o, rtol=1e-4)
 
 
+@pytest.mark.parametrize("n", [1, 40])
+@pytest.mark.parametrize("nx,ny,sx,sy,k,reg", [
+    (48, 48, 48, 48, 11, REG_LAPLACIAN),
+    (48, 40, 33, 31, 3, REG_IDENTITY),
+    (64, 64, 60, 62, 21, REG_LAPLACIAN),  # more rays than are staged
+    (96, 83, 70, 61, 7, REG_GRADIENT),
+])
+def test_cluster_sources_as_fine_as_the_image(mods, ctx32, n, nx, ny, sx, sy, k, reg):
+    # the cluster kernel's ray-by-ray form of L^T against the general kernel's (variant 4)
+    g = Geometry(nx, ny, 3.2 / max(nx, ny), sx, sy, -0.8, 0.8, -0.8, 0.8, k, 1, reg)
+    p = device_problem(make_problem(g, seed=8, psf_sigma=max(k / 6.0, 0.5)))
+    lens = _lens_t(synth.lens_population(np.random.default_rng(9), n))
+    lams = synth.lambda_grid(3, 1.0, 1e2)
+    run = lambda v: ctx32.eval_batch([p], lens, [0] * n, _lam_t(lams, n), [3] * n, want_all_x=True, variant=v)
+    a, b = run(0), run(4)
+    for key in KEYS:
+        assert torch.equal(a[key], b[key]), key
+
+
 @pytest.mark.parametrize("n", [1, 24])
 @pytest.mark.parametrize("nx,ny,sx,sy,k", [(32, 32, 16, 16, 13), (24, 20, 9, 24, 13), (28, 36, 24, 17, 15)])
 def test_cluster_few_rays(mods, nx, ny, sx, sy, k, n):
