@@ -361,7 +361,10 @@ struct ClusterPlan {
 //   48 48 11: 43, 90, 55, 42, 33   48 32 15: 34, 47, 33, 25, 23
 //   64 32 15: 37, 55, 34, 28, 23   96 48 11: (96), 76, 48, 38, 30
 //   128 48 15: (172), -, 99, 78, 57   256 128 21: (1555), -, -, -, 159
-// (in brackets: not all in shared memory).  A source about as fine as the image
+// (in brackets: not all in shared memory; there the time of a loaded device
+// counts, where the slabs' traffic adds up: 2048 items at 256 x 256 and K = 21 took
+// 1155 of SM time an iteration with two CTAs an SM, and clusters of eight, of which
+// 15 fit the 152 SMs, 1611).  A source about as fine as the image
 // has its L^T summed ray by ray (`gather`), which costs both kernels clocks per
 // source pixel.  The two-CTA kernel: 27.5 each of two at 64 x 64, K = 9.
 struct IterCost {
@@ -373,17 +376,19 @@ IterCost fast_cost(const Prob<T>& P) {
     return {2.0 * c, c};
 }
 template <typename T>
-IterCost general_cost(const Prob<T>& P, bool in_smem) {
+IterCost general_cost(const Prob<T>& P, int place) {
     if (P.fft_m) return {6.0 * P.fft_m * P.fft_m, 6.0 * P.fft_m * P.fft_m};
     const int per = (P.ntiles + NTHREADS - 1) / NTHREADS;
     double c = 14500.0 + 73.0 * P.K * P.K * per + 1.5 * P.nrays + (4 * P.ncells > P.plen ? 7.2 * P.ns : 0.0);
-    if (!in_smem) c *= 1.6;
-    return {c, c};
+    if (place == PLACE_SMEM || place == PLACE_SMEM2) return {c, c};
+    c = 11.7 * P.nrays + 111.0 * P.K * P.K * per;
+    if (layout_of(place) == PLACE_MID) return {0.58 * c, 0.84 * c};
+    return {c, two_per_sm(place) ? 0.75 * c : c};
 }
 inline IterCost cluster_cost(const Prob<float>& P, int C, int nt) {
     const double conv = 4.0 * P.K * P.K * P.npix, rays = P.nrays;
     const double lat = 20000.0 + 0.6 * rays + (conv / 170.0 + 3.5 * rays + (4 * P.ncells > P.plen ? 25.0 * P.ns : 0.0)) / C;
-    return {lat, lat * C * (nt > NTHREADS ? 1.0 : 0.85)};
+    return {lat, lat * C * (nt > NTHREADS ? 1.0 : 0.85) * (C == 8 ? 1.27 : 1.0)};
 }
 
 // dynamic shared memory of a cluster-kernel CTA: two CTAs of 256 threads share
@@ -832,25 +837,32 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         ClusterPlan cp;  // C = 0: general kernel
     };
     std::vector<Form> cheap(n_probs), quick(n_probs);
+    std::vector<double> whole(n_probs, 0.0);  // > 0: one form for all items, chosen for this weight
     double limit = 0.0;     // clocks that an item may take in its problem's cheap form
     double call_time = 0.0;  // estimated clocks of the call
     // form of an item of problem p with w iterations where items may take T_ clocks
     auto form_of = [&](int p, double w, double T_) -> const Form& {
+        if (whole[p] > 0.0) w = whole[p];
         return w * cheap[p].it.lat > T_ && quick[p].it.lat < 0.8 * cheap[p].it.lat ? quick[p] : cheap[p];
     };
     {
         std::map<std::pair<int, int>, int> classes;  // (problem, lambdas) -> candidates
-        for (int c = 0; c < n_cand; ++c) classes[{prob_idx[c], n_lam[c]}]++;
+        std::vector<double> longest_w(n_probs, 0.0);
+        for (int c = 0; c < n_cand; ++c) {
+            classes[{prob_idx[c], n_lam[c]}]++;
+            longest_w[prob_idx[c]] = std::max(longest_w[prob_idx[c]], chain_weight(n_lam[c], 0));
+        }
         for (int p = 0; p < n_probs; ++p) {
             if (!cands_of[p]) continue;
             int m = 0;
             bool f = false;
             const bool fast_p = choose(hp[p], m, f) != nullptr;
-            cheap[p].it = fast_p ? fast_cost(hp[p]) : general_cost(hp[p], pick_place<T>(ctx, hp[p], o.place) == PLACE_SMEM);
+            cheap[p].it = fast_p ? fast_cost(hp[p]) : general_cost(hp[p], pick_place<T>(ctx, hp[p], o.place));
             quick[p] = cheap[p];
             if constexpr (sizeof(T) == 4) {
                 if (fast_p || o.place != 0 || want == 4 || want == 5 || want == 6) continue;
-                bool any = pick_place<T>(ctx, hp[p]) == PLACE_SMEM;
+                const bool in_smem = pick_place<T>(ctx, hp[p]) == PLACE_SMEM;
+                bool any = in_smem;
                 for (int C = 1; C <= CL_MAX; C *= 2) {
                     Form x;
                     if (!cluster_fits<T>(ctx, hp[p], C, x.cp)) continue;
@@ -858,6 +870,13 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                     if (!any || x.it.thr < cheap[p].it.thr) cheap[p] = x;
                     if (!any || x.it.lat < quick[p].it.lat) quick[p] = x;
                     any = true;
+                }
+                // the general kernel on its slabs where its work a device is less; all
+                // items of the problem or none, since its CTAs would hold up clusters
+                const IterCost g = general_cost(hp[p], pick_place<T>(ctx, hp[p]));
+                if (any && !in_smem && g.thr < cheap[p].it.thr) {
+                    cheap[p] = Form{g, ClusterPlan()};
+                    whole[p] = longest_w[p];
                 }
             }
         }
