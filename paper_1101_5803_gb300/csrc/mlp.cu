@@ -440,7 +440,11 @@ struct Buf {
         if (p) cudaFree(p);
         p = nullptr;
         n = 0;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) return mlp_fail(MIRAGE_ERR_NOMEM, "mlp: cudaMalloc failed");
+        if (cudaMalloc(&p, bytes) != cudaSuccess) {
+            p = nullptr;
+            cudaGetLastError();  // (reported here, not by a later launch's check)
+            return mlp_fail(MIRAGE_ERR_NOMEM, "mlp: cudaMalloc failed");
+        }
         n = bytes;
         return MIRAGE_OK;
     }
@@ -484,18 +488,20 @@ constexpr int layer_smem() {
 int ensure_batch(mirage_mlp* m, int n) {
     if (n <= m->cap_rows) return MIRAGE_OK;
     long zt = 0, at = 0;
-    m->z_off.assign(m->L + 1, 0);
-    m->a_off.assign(m->L + 1, 0);
+    std::vector<long> z_off(m->L + 1, 0), a_off(m->L + 1, 0);
     int maxw = 0;
     for (int l = 0; l <= m->L; ++l) {
-        m->a_off[l] = at;
+        a_off[l] = at;
         at += ((long)n * m->dims[l] + 7) & ~7L;  // (16-byte rows stay aligned)
         maxw = std::max(maxw, m->dims[l]);
         if (l > 0) {
-            m->z_off[l] = zt;
+            z_off[l] = zt;
             zt += (long)n * m->dims[l];
         }
     }
+    // A buffer that fails to grow is gone, and others have grown by then: no batch
+    // fits until all are there, and the offsets change with the capacity
+    m->cap_rows = 0;
     int r;
     if ((r = m->Z.ensure(sizeof(float) * zt))) return r;
     if ((r = m->A.ensure(sizeof(__nv_bfloat16) * at))) return r;
@@ -503,6 +509,8 @@ int ensure_batch(mirage_mlp* m, int n) {
     if ((r = m->DZH.ensure(2 * sizeof(__nv_bfloat16) * (((long)n * maxw + 7) & ~7L)))) return r;
     if ((r = m->DA.ensure(sizeof(float) * (long)n * maxw))) return r;
     if ((r = m->LOSS.ensure(sizeof(double)))) return r;
+    m->z_off = z_off;
+    m->a_off = a_off;
     m->maxw = maxw;
     m->cap_rows = n;
     return MIRAGE_OK;
