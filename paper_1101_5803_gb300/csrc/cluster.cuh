@@ -497,12 +497,15 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 PA[i] = 0.f;
                 PB[i] = i < n ? I.swp[g0 + i] : 0.f;  // sqrt(W) of the band and its halo, for the preconditioner
             }
-            // zero frames of the FP64 images
+            // the FP64 images outside the tiles that are convolved: zeros in L x, and zero
+            // times the data in the weighted residuals, which is a NaN, as it is in k_cgls,
+            // at an unusable pixel whose value is not finite
             const int part = (g.plen + (int)C - 1) / (int)C, i1 = min((int)(rank + 1) * part, g.plen);
             for (int i = rank * part + tid; i < i1; i += NT) {
+                const double z = 0.0 * (double)I.dpad[i];
                 I.Pa[i] = 0.0;
-                I.Pb[i] = 0.0;
-                I.Rs[i] = 0.0;
+                I.Pb[i] = z;
+                I.Rs[i] = z;
             }
         }
         cl_sync();  // (a slice may lie in another CTA's band)
@@ -633,7 +636,6 @@ __global__ void __launch_bounds__(NT, 2 * NTHREADS / NT) k_cgls_cluster(CglsArgs
                 for (int t = v; t < nt; t += VT) {
                     int ty, tx;
                     tile_at(t, ty, tx);
-                    if (ty < I.tyA || ty >= I.tyB) continue;  // zeros
                     const double* q = I.Rs + (ty * TILE + HK) * Wp + tx * TILE + g.xoff;
                     double r[16];
 #pragma unroll
