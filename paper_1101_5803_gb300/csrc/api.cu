@@ -1145,7 +1145,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     const KernelTable& tb = table();
 
     for (Group* g : glist) TRY(set_smem(ctx, g->fn, g->smem));
-    if (spec_stride) TRY(set_smem(ctx, tb.psf_spectra[prec], fft_smem_bytes(1024)));
+    if (spec_stride) TRY(set_smem(ctx, tb.psf_spectra[prec], fft_smem_bytes(1024, false)));
     TRY(set_smem(ctx, tb.raytrace[prec], (size_t)max_cells * 4));
     if (4 * (max_cells + max_rays) <= ctx->max_smem - 2048) TRY(set_smem(ctx, tb.rt_cells[prec], sizeof(int) * (size_t)(max_cells + max_rays)));
     TRY(set_smem(ctx, tb.rt_place[prec], (size_t)max_cells * 4));
@@ -1196,7 +1196,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     int rc = MIRAGE_OK;
     if (spec_stride) {  // PSF spectra of the FFT problems (once per call)
         void* sa[] = {(void*)&dprobs, (void*)&d_spec64, (void*)&d_spec32, (void*)&spec_stride};
-        rc = launch(ctx, tb.psf_spectra[prec], dim3(n_probs), dim3(NTHREADS), sa, fft_smem_bytes(1024), st);
+        rc = launch(ctx, tb.psf_spectra[prec], dim3(n_probs), dim3(NTHREADS), sa, fft_smem_bytes(1024, false), st);
     }
     do {
         if (rc) break;

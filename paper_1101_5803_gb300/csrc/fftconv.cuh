@@ -39,9 +39,12 @@ constexpr int FFT_BUF_BYTES = 64 * 1024;  // shared ping-pong buffers of one bat
 // half spectrum in shared memory (fftshared.cuh): rows of M + 1 points, and
 // one exchange buffer of M + M / 16 points for each of the 256 threads' transforms
 __host__ __device__ constexpr bool fft_shared(int M) { return M == 64 || M == 128; }
-// batch buffers of size-M plans (bytes), for CTAs of 256 threads
-__host__ __device__ constexpr int fft_buf_bytes(int M) {
-    return fft_shared(M) && 8 * ((M / 2 + 1) * (M + 1) + 256 * 16 / M * (M + M / 16)) > FFT_BUF_BYTES
+// buffers of size-M plans (bytes), for CTAs of 256 threads: the batches', and in
+// single precision what the form of fftshared.cuh takes where that is more
+// (M = 128: 99.5 KB).  Double precision has the batches alone, and at K = 65 no
+// room for more: 211 KB with them, taps included, of 227 KB
+__host__ __device__ constexpr int fft_buf_bytes(int M, bool single) {
+    return single && fft_shared(M) && 8 * ((M / 2 + 1) * (M + 1) + 256 * 16 / M * (M + M / 16)) > FFT_BUF_BYTES
                ? 8 * ((M / 2 + 1) * (M + 1) + 256 * 16 / M * (M + M / 16))
                : FFT_BUF_BYTES;
 }
@@ -64,10 +67,11 @@ __host__ __device__ inline int fft_size_for(int n) {
     return m;
 }
 
-// shared bytes of the FFT path for size M: two plans, both twiddle tables
-// (with alignment slack) and the batch buffers
-__host__ __device__ inline size_t fft_smem_bytes(int M) {
-    return 128 + (size_t)(M - 1) * (sizeof(float2) + sizeof(double2)) + 64 + fft_buf_bytes(M);
+// shared bytes of the FFT path for size M in a context of single or double
+// precision: two plans, both twiddle tables (with alignment slack) and the
+// buffers
+__host__ __device__ inline size_t fft_smem_bytes(int M, bool single) {
+    return 128 + (size_t)(M - 1) * (sizeof(float2) + sizeof(double2)) + 64 + fft_buf_bytes(M, single);
 }
 
 // transforms per batch for element type C

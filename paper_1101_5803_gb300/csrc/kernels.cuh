@@ -1558,7 +1558,7 @@ __host__ __device__ inline size_t smem_bytes(const Prob<T>& P, int place) {
         o += 4 * align_up<T>(sizeof(T) * P.ns, 16);                    // x p s minv
         o += 2 * align_up<T>(sizeof(T) * P.nreg, 16);                  // rreg qreg
     }
-    if (P.fft_m) o += fft_smem_bytes(P.fft_m);                         // FFT twiddles and batch buffers
+    if (P.fft_m) o += fft_smem_bytes(P.fft_m, sizeof(T) == 4);         // FFT twiddles and buffers
     return o;
 }
 
