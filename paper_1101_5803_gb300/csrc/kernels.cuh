@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "cellsort.cuh"
 #include "dfloat.cuh"
 #include "fftconv.cuh"
 #include "fftshared.cuh"
@@ -448,6 +449,9 @@ __global__ void __launch_bounds__(NTHREADS) k_raytrace(const Prob<T>* __restrict
 // shared memory, then one pass over the rays.  The same arrays as k_raytrace.
 // ---------------------------------------------------------------------------
 constexpr int RT_THREADS = 128, RT_PLACE_THREADS = 1024;
+// rays of a cell that one thread, and that one warp sorts; longer ones fill at
+// most this many of the 58112 numbers that shared memory holds (227 KB)
+constexpr int RT_CELL_THREAD = 32, RT_CELL_WARP = 1024, RT_LONG_CELLS = 58112 / RT_CELL_WARP + 1;
 
 template <typename T>
 __global__ void __launch_bounds__(RT_THREADS) k_rt_rays(const Prob<T>* __restrict__ probs,
@@ -486,7 +490,7 @@ __global__ void __launch_bounds__(RT_PLACE_THREADS) k_rt_cells(const Prob<T>* __
     const int c = cand0 + blockIdx.x;
     const Prob<T>& P = probs[cand_prob[c]];
     extern __shared__ int sh_counts[];  // [ncells] counts, then ends; [nrays] ray numbers by cell
-    __shared__ int s_warp[RT_PLACE_THREADS / 32], s_active;
+    __shared__ int s_warp[RT_PLACE_THREADS / 32], s_active, s_nlong, s_long[RT_LONG_CELLS];
     int* list = sh_counts + P.ncells;
     const int tid = threadIdx.x, lane = tid & 31, bs = RT_PLACE_THREADS;
     if (make_lens<double>(lens + 7LL * c).bad) {
@@ -500,7 +504,10 @@ __global__ void __launch_bounds__(RT_PLACE_THREADS) k_rt_cells(const Prob<T>* __
     int* cst = cs.cst + (long long)c * cs.sCst;
     const T* swp = cs.swp + (long long)c * cs.sPad;
     for (int i = tid; i < P.ncells; i += bs) sh_counts[i] = 0;
-    if (tid == 0) s_active = 0;
+    if (tid == 0) {
+        s_active = 0;
+        s_nlong = 0;
+    }
     __syncthreads();
     auto cell_of = [&](int base) {
         const int iy0 = base / P.sx;
@@ -559,19 +566,38 @@ __global__ void __launch_bounds__(RT_PLACE_THREADS) k_rt_cells(const Prob<T>* __
             inv[r] = -1;
     }
     __syncthreads();
-    for (int i = tid; i < P.ncells; i += bs) {  // insertion sort (cells hold few rays)
-        const int k0 = i > 0 ? sh_counts[i - 1] : 0, k1 = sh_counts[i];
-        for (int a = k0 + 1; a < k1; ++a) {
-            const int key = list[a];
-            int b = a - 1;
-            while (b >= k0 && list[b] > key) {
-                list[b + 1] = list[b];
-                --b;
+    // Each cell back into ray order.  Most cells hold a few rays in nearly that
+    // order: an insertion sort by one thread.  That takes up to n^2 / 4 dependent
+    // moves for n rays, and a coarse source or sub-pixel rays put thousands into a
+    // cell (64 x 64 pixels of 2 x 2 rays on a 2 x 2 source: 16384 in one, and 226 ms
+    // for a call that takes 22), so longer cells are sorted by a warp and the longest
+    // by all of them
+    for (int i0 = tid - lane; i0 < P.ncells; i0 += bs) {
+        const int i = i0 + lane, k0 = i < P.ncells && i > 0 ? sh_counts[i - 1] : 0, k1 = i < P.ncells ? sh_counts[i] : k0;
+        if (k1 - k0 <= RT_CELL_THREAD) {
+            for (int a = k0 + 1; a < k1; ++a) {
+                const int key = list[a];
+                int b = a - 1;
+                while (b >= k0 && list[b] > key) {
+                    list[b + 1] = list[b];
+                    --b;
+                }
+                list[b + 1] = key;
             }
-            list[b + 1] = key;
+        } else if (k1 - k0 > RT_CELL_WARP) {
+            s_long[atomicAdd(&s_nlong, 1)] = i;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, k1 - k0 > RT_CELL_THREAD && k1 - k0 <= RT_CELL_WARP);
+        for (; todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1, q0 = __shfl_sync(0xffffffffu, k0, src), q1 = __shfl_sync(0xffffffffu, k1, src);
+            cell_sort(list + q0, q1 - q0, lane, 32, [] { __syncwarp(); });
         }
     }
     __syncthreads();
+    for (int j = 0; j < s_nlong; ++j) {
+        const int i = s_long[j], k0 = i > 0 ? sh_counts[i - 1] : 0;
+        cell_sort(list + k0, sh_counts[i] - k0, tid, bs, [] { __syncthreads(); });
+    }
     const int n = P.ncells > 0 ? sh_counts[P.ncells - 1] : 0;
     for (int p = tid; p < n; p += bs) {
         const int r = list[p];
