@@ -1185,7 +1185,10 @@ enum : int { CONV_Q = 0, CONV_RAW = 1 };
 // taps[a][b] Pb[a Wp + c + b + sh], terms in the order a, b.  Small images have
 // fewer 4 x 4 tiles than a CTA has threads (64 of 256 at 32 x 32), and the FP64
 // units of the idle warps' SM sub-partitions would stand still; a row a thread
-// keeps them all busy.
+// keeps them all busy.  Taken up to 128 tiles, where the gain ends: 160
+// candidates x 8 lambdas at K = 9 took 211 ms by tiles and 98.6 by rows at 32 x 32
+// (64 tiles), 211 and 157 at 36 x 36 (81), 214 and 188 at 44 x 44 (121), 258
+// and 229 at 64 x 32 (128); K = 5 at 121 and 128 tiles: no difference.
 __device__ __forceinline__ void conv_row64(const double* __restrict__ Pb, int Wp, const double* __restrict__ taps, int K,
                                            int KP, double (&acc)[TILE]) {
 #pragma unroll
@@ -1212,6 +1215,36 @@ __device__ __forceinline__ bool conv_by_rows(const Geo<T>& g) {
     return sizeof(T) == 8 && 2 * g.ntiles <= (int)blockDim.x;
 }
 
+// conv_pass by rows
+template <int K>
+__device__ __noinline__ double conv_rows_pass(const double* __restrict__ src, const double* __restrict__ taps,
+                                              const double* __restrict__ swp, double* __restrict__ dst, Geo<double> g,
+                                              int mode) {
+    double ss = 0;
+    const int kk = K > 0 ? K : g.K, kp = K > 0 ? (K + 3) & ~3 : g.kp;
+    for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
+        const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
+        double acc[TILE];
+        conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, kk, kp, acc);
+        const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
+#pragma unroll
+        for (int c = 0; c < TILE; ++c) dst[pp + c] = mode == CONV_Q ? swp[pp + c] * acc[c] : acc[c];
+    }
+    if (mode == CONV_Q) {  // the sum in the order of the tiles' owners
+        __syncthreads();
+        for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
+            const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
+#pragma unroll
+            for (int r = 0; r < TILE; ++r) {
+                const V4<double> o = ld4(dst + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) ss = fma(o.v[c], o.v[c], ss);
+            }
+        }
+    }
+    return ss;
+}
+
 // One convolution over all owned tiles (one non-inlined copy of the
 // unrolled tile code per kernel):
 //   CONV_Q   : dst = sqrt(W) * conv, returns sum dst^2
@@ -1220,32 +1253,6 @@ template <typename T, int K, bool SH>
 __device__ __noinline__ T conv_pass(const T* __restrict__ src, const T* __restrict__ taps,
                                          const T* __restrict__ swp, T* __restrict__ dst, Geo<T> g, int mode) {
     T ss = 0;
-    if constexpr (sizeof(T) == 8) {
-        if (conv_by_rows(g)) {
-            const int kk = K > 0 ? K : g.K, kp = K > 0 ? (K + 3) & ~3 : g.kp;
-            for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
-                const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
-                double acc[TILE];
-                conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, kk, kp, acc);
-                const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
-#pragma unroll
-                for (int c = 0; c < TILE; ++c) dst[pp + c] = mode == CONV_Q ? swp[pp + c] * acc[c] : acc[c];
-            }
-            if (mode == CONV_Q) {  // the sum in the order of the tiles' owners
-                __syncthreads();
-                for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
-                    const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-#pragma unroll
-                    for (int r = 0; r < TILE; ++r) {
-                        const V4<T> o = ld4(dst + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) ss = fma(o.v[c], o.v[c], ss);
-                    }
-                }
-            }
-            return ss;
-        }
-    }
     for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
         const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
         T acc[TILE][TILE];
@@ -1275,6 +1282,16 @@ __device__ __noinline__ T conv_pass(const T* __restrict__ src, const T* __restri
     return ss;
 }
 
+// the direct convolution of an image, by rows or by tiles (each a function of
+// its own: with both in one, FP64 images of more than 128 tiles lost 1% to the
+// rows' registers)
+template <typename T, int K, bool SH>
+__device__ __forceinline__ T conv_direct(const T* src, const T* taps, const T* swp, T* dst, const Geo<T>& g, int mode) {
+    if constexpr (sizeof(T) == 8)
+        if (conv_by_rows(g)) return conv_rows_pass<K>(src, taps, swp, dst, g, mode);
+    return conv_pass<T, K, SH>(src, taps, swp, dst, g, mode);
+}
+
 // FP64 convolution pass of the refinement:
 //   mode 0: res = sqrt(W)(d - conv(Pa)); rimg = (T)res; Pb = sqrt(W) res; returns sum res^2
 //   mode 1: Pc = conv(Pb)
@@ -1301,40 +1318,6 @@ __device__ __noinline__ double conv64_pass(const Work<T> w, Geo<T> g, int mode) 
     }
     const double* src = mode == 0 ? w.Pa : w.Pb;
     const double* taps = w.taps64 + (mode == 0 ? 0 : g.K * g.kp);
-    if (sizeof(T) == 8 && conv_by_rows(g)) {  // (Pc holds the residuals until their sum is taken)
-        for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
-            const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
-            double acc[TILE];
-            conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, g.K, g.kp, acc);
-            const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
-#pragma unroll
-            for (int c = 0; c < TILE; ++c) {
-                if (mode == 0) {
-                    const double sw = (double)w.swp[pp + c];
-                    const double res = sw * ((double)w.dpad[pp + c] - acc[c]);
-                    w.rimg[pp + c] = (T)res;
-                    w.Pb[pp + c] = sw * res;
-                    w.Pc[pp + c] = res;
-                } else {
-                    w.Pc[pp + c] = acc[c];
-                }
-            }
-        }
-        if (mode == 0) {
-            __syncthreads();
-            for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
-                const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-#pragma unroll
-                for (int r = 0; r < TILE; ++r) {
-                    const V4<double> o = ld4(w.Pc + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) ss += o.v[c] * o.v[c];
-                }
-            }
-            __syncthreads();
-        }
-        return ss;
-    }
     for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
         const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
         double acc[TILE][TILE];
@@ -1476,6 +1459,46 @@ __device__ __noinline__ double conv64_df_gen(const double* __restrict__ src, flo
     return ss;
 }
 
+// conv64_pass by rows (Pc holds the residuals until their sum is taken)
+template <typename T>
+__device__ __noinline__ double conv64_rows_pass(const Work<T> w, Geo<T> g, int mode) {
+    double ss = 0;
+    const double* src = mode == 0 ? w.Pa : w.Pb;
+    const double* taps = w.taps64 + (mode == 0 ? 0 : g.K * g.kp);
+    for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
+        const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
+        double acc[TILE];
+        conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, g.K, g.kp, acc);
+        const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
+#pragma unroll
+        for (int c = 0; c < TILE; ++c) {
+            if (mode == 0) {
+                const double sw = w.swp[pp + c];
+                const double res = sw * (w.dpad[pp + c] - acc[c]);
+                w.rimg[pp + c] = res;
+                w.Pb[pp + c] = sw * res;
+                w.Pc[pp + c] = res;
+            } else {
+                w.Pc[pp + c] = acc[c];
+            }
+        }
+    }
+    if (mode == 0) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
+            const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
+#pragma unroll
+            for (int r = 0; r < TILE; ++r) {
+                const V4<double> o = ld4(w.Pc + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) ss += o.v[c] * o.v[c];
+            }
+        }
+        __syncthreads();
+    }
+    return ss;
+}
+
 // the general kernel's refinement passes: double-float for direct
 // convolution in FP32 contexts, conv64_pass otherwise (FP64 contexts, FFT)
 template <typename T, int KT>
@@ -1486,6 +1509,8 @@ struct Conv64Gen {
                 return conv64_df_gen<KT>(mode == 0 ? w.Pa : w.Pb, w.P1, w.P2, w.taps + (mode == 0 ? 0 : g.K * g.kp),
                                          w.swp, w.dpad, w.rimg, w.Pb, w.Pc, g, mode);
         }
+        if constexpr (sizeof(T) == 8)
+            if (!w.fft && conv_by_rows(g)) return conv64_rows_pass<T>(w, g, mode);
         return conv64_pass<T>(w, g, mode);
     }
 };
@@ -2007,9 +2032,9 @@ __global__ void __launch_bounds__(NTHREADS, MINB) k_cgls(CglsArgs<T> A) {
                 T cq;
                 if constexpr (K == 0 && BIG)
                     cq = w.fft ? conv_pass_fft<T>(&w.fft->t, w.P1, w.swp, w.qimg, g, CONV_Q)
-                               : conv_pass<T, K, SH>(w.P1, w.taps, w.swp, w.qimg, g, CONV_Q);
+                               : conv_direct<T, K, SH>(w.P1, w.taps, w.swp, w.qimg, g, CONV_Q);
                 else
-                    cq = conv_pass<T, K, SH>(w.P1, w.taps, w.swp, w.qimg, g, CONV_Q);
+                    cq = conv_direct<T, K, SH>(w.P1, w.taps, w.swp, w.qimg, g, CONV_Q);
                 {
                     const double delta = block_sum_to0<T>(cq + lamT * dh, red);
                     if (tid == 0) {
@@ -2043,9 +2068,9 @@ __global__ void __launch_bounds__(NTHREADS, MINB) k_cgls(CglsArgs<T> A) {
                     if (w.fft)
                         conv_pass_fft<T>(&w.fft->t, w.P2, nullptr, w.qimg, g, CONV_RAW);
                     else
-                        conv_pass<T, K, SH>(w.P2, w.taps + g.K * g.kp, nullptr, w.qimg, g, CONV_RAW);
+                        conv_direct<T, K, SH>(w.P2, w.taps + g.K * g.kp, nullptr, w.qimg, g, CONV_RAW);
                 } else {
-                    conv_pass<T, K, SH>(w.P2, w.taps + g.K * g.kp, nullptr, w.qimg, g, CONV_RAW);
+                    conv_direct<T, K, SH>(w.P2, w.taps + g.K * g.kp, nullptr, w.qimg, g, CONV_RAW);
                 }
                 __syncthreads();  // u complete
                 // (A p)_i = (L^T u)_i + lam (H^T H p)_i, then the CG updates of
