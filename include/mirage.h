@@ -276,6 +276,15 @@ int mirage_set_reserved_slots(mirage_ctx_t* ctx, int slots);
  * issued (a replayed graph counts its kernels). */
 int mirage_last_launch_count(const mirage_ctx_t* ctx);
 
+/* Which kernel ran the items of the last mirage_eval_batch on this context (an
+ * item is one candidate at one lambda):
+ *  out[0]     the two-CTA kernel
+ *  out[1]     the general kernel, direct convolution
+ *  out[2]     the general kernel, convolution by FFT
+ *  out[3..6]  the cluster kernel on 1, 2, 4 and 8 SMs */
+#define MIRAGE_N_ITEM_KERNELS 7
+int mirage_last_item_kernels(const mirage_ctx_t* ctx, int* out);
+
 /* Device time (ms) of the three phases of the last batched, non-graph call
  * made with opts->threads < 0: ms[0] ray trace, ms[1] CGLS items, ms[2]
  * L-curve/finalize.  Waits for those events. */

@@ -92,6 +92,8 @@ def load_library():
     lib.mirage_set_reserved_slots.restype = ip
     lib.mirage_last_launch_count.argtypes = [vp]
     lib.mirage_last_launch_count.restype = ip
+    lib.mirage_last_item_kernels.argtypes = [vp, ctypes.POINTER(i)]
+    lib.mirage_last_item_kernels.restype = ip
     lib.mirage_last_phase_clocks.argtypes = [vp, vp]
     lib.mirage_last_phase_clocks.restype = ip
     lib.mirage_last_phase_ms.argtypes = [vp, vp]
@@ -190,6 +192,16 @@ def mirage_destroy(ctx) -> None:
 
 def mirage_last_launch_count(ctx) -> int:
     return int(load_library().mirage_last_launch_count(ctx))
+
+
+ITEM_KERNELS = ("two_cta", "direct", "fft", "cluster1", "cluster2", "cluster4", "cluster8")
+
+
+def mirage_last_item_kernels(ctx) -> dict:
+    """Items of the last evaluation by the kernel that ran them (mirage.h)."""
+    buf = (ctypes.c_int * len(ITEM_KERNELS))()
+    _check(load_library().mirage_last_item_kernels(ctx, buf), "mirage_last_item_kernels")
+    return dict(zip(ITEM_KERNELS, buf))
 
 
 def mirage_eval_batch(ctx, probs, lens, prob_idx, lambdas, n_lam, *, tol=1e-6, maxit=0,
@@ -464,6 +476,9 @@ class Context:
 
     def launches(self) -> int:
         return mirage_last_launch_count(self.handle)
+
+    def item_kernels(self) -> dict:
+        return mirage_last_item_kernels(self.handle)
 
     def phase_ms(self):
         return mirage_last_phase_ms(self.handle)

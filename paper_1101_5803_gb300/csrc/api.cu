@@ -117,6 +117,7 @@ struct mirage_ctx {
     int max_smem = 0;
     int max_smem_sm = 0;
     int last_launches = 0;
+    int last_kernels[MIRAGE_N_ITEM_KERNELS] = {};  // items of the last evaluation by kernel
     int reserved = 0;  // CTA slots the CGLS launches leave free (mirage_set_reserved_slots)
     // scratch
     DevBuf E, E64, Etmp, inv, cst, swp, dpad, nent, cstat, X, istat, slab, probs, cand_prob, items, counters;
@@ -894,11 +895,13 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         }
         for (double T_ = 0.5 * total; T_ < 1e3 * total; T_ *= 1.5) {
             double sum = 0.0, longest = 0.0;
+            bool other = false;  // items in their second form
             for (auto& x : classes)
                 for (double wk : w[x.first.second]) {
-                    const IterCost& it = form_of(x.first.first, wk, T_).it;
-                    sum += x.second * wk * it.thr / ctx->sm_count;
-                    longest = std::max(longest, wk * it.lat);
+                    const Form& form = form_of(x.first.first, wk, T_);
+                    sum += x.second * wk * form.it.thr / ctx->sm_count;
+                    longest = std::max(longest, wk * form.it.lat);
+                    other |= whole[x.first.first] == 0.0 && &form == &quick[x.first.first];
                 }
             const double est = std::max(sum, longest) + 0.5 * std::min(sum, longest);
             if (est < 0.98 * best) {
@@ -906,7 +909,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                 limit = T_;
                 call_time = std::max(sum, longest);
             }
-            if (!two || longest < T_) break;  // a larger limit changes nothing more
+            if (!two || !other) break;  // every item in the first form: a larger limit changes nothing more
         }
         if (o.mode == MIRAGE_MODE_PLAIN) limit = 0.0;  // one candidate at a time
     }
@@ -921,6 +924,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         }
         chain_budget = tw / (double)cgls_slots(ctx, 2);
     }
+    std::fill(ctx->last_kernels, ctx->last_kernels + MIRAGE_N_ITEM_KERNELS, 0);
     for (int c = 0; c < n_cand; ++c) {
         const Prob<T>& P = hp[prob_idx[c]];
         int place = pick_place<T>(ctx, P, o.place);
@@ -962,6 +966,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
             g.slab = std::max<long long>(g.slab, cp.C ? cp.slab : item_slab);
             g.load += form.it.lat * chain_weight(n_lam[c], k);
             g.longest = std::max(g.longest, form.it.lat * w);
+            ++ctx->last_kernels[cp.C ? 3 + (cp.C > 1) + (cp.C > 2) + (cp.C > 4) : fast ? 0 : P.fft_m ? 2 : 1];
             return &g;
         };
         for (int k = n_lam[c] - 1; k > 0; --k)
@@ -1703,6 +1708,12 @@ int mirage_set_reserved_slots(mirage_ctx_t* ctx, int slots) {
 }
 
 int mirage_last_launch_count(const mirage_ctx_t* ctx) { return ctx ? ctx->last_launches : 0; }
+
+int mirage_last_item_kernels(const mirage_ctx_t* ctx, int* out) {
+    if (!ctx || !out) return MIRAGE_ERR_ARG;
+    std::copy(ctx->last_kernels, ctx->last_kernels + MIRAGE_N_ITEM_KERNELS, out);
+    return MIRAGE_OK;
+}
 
 static_assert(MAX_LAM == MIRAGE_MAX_LAM, "lambda grid limit of the header and the kernels");
 
