@@ -774,7 +774,6 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     std::vector<int> cls_of(n_probs);
     struct Group {
         const void* fn;
-        bool big;
         bool fast = false;
         int cl = 0, nt = NTHREADS;  // cluster kernel: CTAs per item, threads a CTA
         int prob = -1;   // the single problem of the group, -2 if several
@@ -835,98 +834,24 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     // kernel and 33 on clusters of four)
     struct Form {
         IterCost it;
-        ClusterPlan cp;  // C = 0: general kernel
+        ClusterPlan cp;  // C = 0: general or two-CTA kernel
     };
-    std::vector<Form> cheap(n_probs), quick(n_probs);
-    std::vector<double> whole(n_probs, 0.0);  // > 0: one form for all items, chosen for this weight
-    double limit = 0.0;     // clocks that an item may take in its problem's cheap form
-    double call_time = 0.0;  // estimated clocks of the call
-    // form of an item of problem p with w iterations where items may take T_ clocks
-    auto form_of = [&](int p, double w, double T_) -> const Form& {
-        if (whole[p] > 0.0) w = whole[p];
-        return w * cheap[p].it.lat > T_ && quick[p].it.lat < 0.8 * cheap[p].it.lat ? quick[p] : cheap[p];
+    // what a problem's items have in common
+    struct ProbPlan {
+        Form cheap, quick;
+        bool whole = false;  // one form for all items
+        const void* fn = nullptr;  // the kernel without clusters, its shared memory, slab, CTAs per SM
+        size_t smem = 0;
+        long long slab = 0;
+        int per_sm = 1, mode = 0;
+        bool fast = false, big = false;
     };
-    {
-        std::map<std::pair<int, int>, int> classes;  // (problem, lambdas) -> candidates
-        std::vector<double> longest_w(n_probs, 0.0);
-        for (int c = 0; c < n_cand; ++c) {
-            classes[{prob_idx[c], n_lam[c]}]++;
-            longest_w[prob_idx[c]] = std::max(longest_w[prob_idx[c]], chain_weight(n_lam[c], 0));
-        }
-        for (int p = 0; p < n_probs; ++p) {
-            if (!cands_of[p]) continue;
-            int m = 0;
-            bool f = false;
-            const bool fast_p = choose(hp[p], m, f) != nullptr;
-            cheap[p].it = fast_p ? fast_cost(hp[p]) : general_cost(hp[p], pick_place<T>(ctx, hp[p], o.place));
-            quick[p] = cheap[p];
-            if constexpr (sizeof(T) == 4) {
-                if (fast_p || o.place != 0 || want == 4 || want == 5 || want == 6) continue;
-                const bool in_smem = pick_place<T>(ctx, hp[p]) == PLACE_SMEM;
-                bool any = in_smem;
-                for (int C = 1; C <= CL_MAX; C *= 2) {
-                    Form x;
-                    if (!cluster_fits<T>(ctx, hp[p], C, x.cp)) continue;
-                    x.it = cluster_cost(hp[p], C, x.cp.nt);
-                    if (!any || x.it.thr < cheap[p].it.thr) cheap[p] = x;
-                    if (!any || x.it.lat < quick[p].it.lat) quick[p] = x;
-                    any = true;
-                }
-                // the general kernel on its slabs where its work a device is less; all
-                // items of the problem or none, since its CTAs would hold up clusters
-                const IterCost g = general_cost(hp[p], pick_place<T>(ctx, hp[p]));
-                if (any && !in_smem && g.thr < cheap[p].it.thr) {
-                    cheap[p] = Form{g, ClusterPlan()};
-                    whole[p] = longest_w[p];
-                }
-            }
-        }
-        // the call's time as a function of the limit: its longest item, or its work
-        // on all SMs, and part of the other one (the end of a call is never packed
-        // full)
-        bool two = false;
-        for (int p = 0; p < n_probs; ++p) two |= quick[p].it.lat < 0.8 * cheap[p].it.lat;
-        std::vector<std::vector<double>> w(max_lam + 1);
-        double total = 0.0, best = 1e300;
-        for (auto& x : classes) {
-            const int n = x.first.second;
-            for (int k = (int)w[n].size(); k < n; ++k) w[n].push_back(chain_weight(n, k));
-            for (int k = 0; k < n; ++k) total += x.second * w[n][k] * cheap[x.first.first].it.thr / ctx->sm_count;
-        }
-        for (double T_ = 0.5 * total; T_ < 1e3 * total; T_ *= 1.5) {
-            double sum = 0.0, longest = 0.0;
-            bool other = false;  // items in their second form
-            for (auto& x : classes)
-                for (double wk : w[x.first.second]) {
-                    const Form& form = form_of(x.first.first, wk, T_);
-                    sum += x.second * wk * form.it.thr / ctx->sm_count;
-                    longest = std::max(longest, wk * form.it.lat);
-                    other |= whole[x.first.first] == 0.0 && &form == &quick[x.first.first];
-                }
-            const double est = std::max(sum, longest) + 0.5 * std::min(sum, longest);
-            if (est < 0.98 * best) {
-                best = est;
-                limit = T_;
-                call_time = std::max(sum, longest);
-            }
-            if (!two || !other) break;  // every item in the first form: a larger limit changes nothing more
-        }
-        if (o.mode == MIRAGE_MODE_PLAIN) limit = 0.0;  // one candidate at a time
-    }
-    // chained calls: each CTA slot's share of the estimated cost of the call
-    double chain_budget = 0.0;
-    if (lam_start) {
-        double tw = 0.0;
-        for (int c = 0; c < n_cand; ++c) {
-            const Prob<T>& P = hp[prob_idx[c]];
-            const double work = (double)P.plen * P.K * P.K + 8.0 * P.nrays;
-            for (int k = 0; k < n_lam[c]; ++k) tw += work * chain_weight(n_lam[c], k);
-        }
-        chain_budget = tw / (double)cgls_slots(ctx, 2);
-    }
-    std::fill(ctx->last_kernels, ctx->last_kernels + MIRAGE_N_ITEM_KERNELS, 0);
-    for (int c = 0; c < n_cand; ++c) {
-        const Prob<T>& P = hp[prob_idx[c]];
+    std::vector<ProbPlan> plan(n_probs);
+    bool second = false;  // some problem has a second form
+    for (int p = 0; p < n_probs; ++p) {
+        if (!cands_of[p]) continue;
+        const Prob<T>& P = hp[p];
+        ProbPlan& q = plan[p];
         int place = pick_place<T>(ctx, P, o.place);
         // FP64, everything in shared memory: two CTAs per SM (128 registers a
         // thread) where two fit and there are many items a slot.  At 32 x 32, 256
@@ -935,48 +860,169 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         if (sizeof(T) == 8 && place == PLACE_SMEM && o.place == 0 && o.mode == MIRAGE_MODE_BATCHED &&
             n_items >= 8LL * ctx->sm_count && 2 * ((long long)smem_bytes<T>(P, PLACE_SMEM) + 1024) <= ctx->max_smem_sm)
             place = PLACE_SMEM2;
-        const bool big = place != PLACE_SMEM;
-        const void* fn = pick_cgls(prec, place, P.fft_m ? 0 : P.K);
-        size_t item_smem = smem_bytes<T>(P, layout_of(place));
-        long long item_slab = (long long)slab_bytes<T>(P, layout_of(place));
-        int per_sm = two_per_sm(place) ? 2 : 1, mode = 0;
-        bool fast = false;
-        if (const void* ff = choose(P, mode, fast)) {
-            fn = ff;
-            item_smem = fast_smem_bytes(*reinterpret_cast<const Prob<float>*>(&P));
-            item_slab = (long long)fast_slab_bytes(*reinterpret_cast<const Prob<float>*>(&P));
-            per_sm = 2;
+        q.big = place != PLACE_SMEM;
+        q.fn = pick_cgls(prec, place, P.fft_m ? 0 : P.K);
+        q.smem = smem_bytes<T>(P, layout_of(place));
+        q.slab = (long long)slab_bytes<T>(P, layout_of(place));
+        q.per_sm = two_per_sm(place) ? 2 : 1;
+        if (const void* ff = choose(P, q.mode, q.fast)) {
+            q.fn = ff;
+            q.smem = fast_smem_bytes(*reinterpret_cast<const Prob<float>*>(&P));
+            q.slab = (long long)fast_slab_bytes(*reinterpret_cast<const Prob<float>*>(&P));
+            q.per_sm = 2;
         }
-        // the group of candidate c's items of lambda k (chains: of the smallest lambda)
-        auto group_of = [&](int k) -> Group* {
-            const double w = chain_weight(n_lam[c], lam_start ? 0 : k);
-            const Form& form = form_of(prob_idx[c], w, limit);
+        q.cheap.it = q.fast ? fast_cost(P) : general_cost(P, pick_place<T>(ctx, P, o.place));
+        q.quick = q.cheap;
+        if constexpr (sizeof(T) == 4) {
+            if (q.fast || o.place != 0 || want == 4 || want == 5 || want == 6) continue;
+            const bool in_smem = pick_place<T>(ctx, P) == PLACE_SMEM;
+            bool any = in_smem;
+            for (int C = 1; C <= CL_MAX; C *= 2) {
+                Form x;
+                if (!cluster_fits<T>(ctx, P, C, x.cp)) continue;
+                x.it = cluster_cost(P, C, x.cp.nt);
+                if (!any || x.it.thr < q.cheap.it.thr) q.cheap = x;
+                if (!any || x.it.lat < q.quick.it.lat) q.quick = x;
+                any = true;
+            }
+            // the general kernel on its slabs where its work a device is less; all
+            // items of the problem or none, since its CTAs would hold up clusters
+            const IterCost g = general_cost(P, pick_place<T>(ctx, P));
+            if (any && !in_smem && g.thr < q.cheap.it.thr) {
+                q.cheap = Form{g, ClusterPlan()};
+                q.whole = true;
+            }
+        }
+        second |= q.quick.it.lat < 0.8 * q.cheap.it.lat;
+    }
+    // candidates of one problem and lambda count are alike: their items' forms and
+    // groups are looked up once, and the weights of an n-point grid made once
+    // (a map look-up and two powers an item took 90 us of a call of 256 x 16)
+    struct Class {
+        int p = 0, n = 0, count = 0;
+        std::vector<const Form*> form;  // by lambda
+        std::vector<Group*> group;
+    };
+    std::map<std::pair<int, int>, Class> classes;
+    std::vector<Class*> class_of(n_cand);
+    std::vector<std::vector<double>> weight(max_lam + 1);
+    for (int c = 0; c < n_cand; ++c) {
+        Class*& cl = class_of[c];
+        if (c > 0 && prob_idx[c] == prob_idx[c - 1] && n_lam[c] == n_lam[c - 1]) {
+            cl = class_of[c - 1];
+        } else {
+            cl = &classes[{prob_idx[c], n_lam[c]}];
+            cl->p = prob_idx[c];
+            cl->n = n_lam[c];
+        }
+        cl->count++;
+        std::vector<double>& w = weight[n_lam[c]];
+        for (int k = (int)w.size(); k < n_lam[c]; ++k) w.push_back(chain_weight(n_lam[c], k));
+    }
+    // form of an item of problem p with w iterations where items may take `limit` clocks
+    auto form_of = [&](const ProbPlan& q, double w, double limit) -> const Form& {
+        return w * q.cheap.it.lat > limit && q.quick.it.lat < 0.8 * q.cheap.it.lat ? q.quick : q.cheap;
+    };
+    auto set_forms = [&](double limit) {
+        for (auto& kv : classes) {
+            Class& cl = kv.second;
+            const ProbPlan& q = plan[cl.p];
+            const std::vector<double>& w = weight[cl.n];
+            cl.form.resize(cl.n);
+            for (int k = 0; k < cl.n; ++k)
+                cl.form[k] = &form_of(q, w[lam_start && o.mode == MIRAGE_MODE_BATCHED ? 0 : k], limit);
+            if (q.whole) std::fill(cl.form.begin(), cl.form.end(), cl.form[0]);
+        }
+    };
+    double call_time = 0.0;  // estimated clocks of the call
+    set_forms(o.mode == MIRAGE_MODE_PLAIN ? 0.0 : 1e300);  // (plain mode: one candidate at a time)
+    if (second && o.mode == MIRAGE_MODE_BATCHED) {
+        // the call's time as a function of the limit: its longest item, or its work
+        // on all SMs, and part of the other one (the end of a call is never packed
+        // full)
+        double total = 0.0, best = 1e300, limit = 1e300;
+        for (auto& kv : classes)
+            for (double wk : weight[kv.second.n]) total += kv.second.count * wk * plan[kv.second.p].cheap.it.thr / ctx->sm_count;
+        for (double T_ = 0.5 * total; T_ < 1e3 * total; T_ *= 1.5) {
+            set_forms(T_);
+            double sum = 0.0, longest = 0.0;
+            bool other = false;  // items in their second form
+            for (auto& kv : classes) {
+                const Class& cl = kv.second;
+                const std::vector<double>& w = weight[cl.n];
+                for (int k = 0; k < cl.n; ++k) {
+                    sum += cl.count * w[k] * cl.form[k]->it.thr / ctx->sm_count;
+                    longest = std::max(longest, w[k] * cl.form[k]->it.lat);
+                    other |= !plan[cl.p].whole && cl.form[k] == &plan[cl.p].quick;
+                }
+            }
+            const double est = std::max(sum, longest) + 0.5 * std::min(sum, longest);
+            if (est < 0.98 * best) {
+                best = est;
+                limit = T_;
+                call_time = std::max(sum, longest);
+            }
+            if (!other) break;  // every item in the first form: a larger limit changes nothing more
+        }
+        set_forms(limit);
+    } else if (plan.size() > 1) {
+        double sum = 0.0, longest = 0.0;
+        for (auto& kv : classes)
+            for (int k = 0; k < kv.second.n; ++k) {
+                const IterCost& it = kv.second.form[k]->it;
+                sum += kv.second.count * weight[kv.second.n][k] * it.thr / ctx->sm_count;
+                longest = std::max(longest, weight[kv.second.n][k] * it.lat);
+            }
+        call_time = std::max(sum, longest);
+    }
+    // groups: items of one kernel (and cluster size) share a launch
+    std::fill(ctx->last_kernels, ctx->last_kernels + MIRAGE_N_ITEM_KERNELS, 0);
+    for (auto& kv : classes) {
+        Class& cl = kv.second;
+        const ProbPlan& q = plan[cl.p];
+        const std::vector<double>& w = weight[cl.n];
+        cl.group.resize(cl.n);
+        for (int k = 0; k < cl.n; ++k) {
+            const Form& form = *cl.form[k];
             const ClusterPlan& cp = form.cp;
-            const void* f = cp.C ? cp.fn : fn;
-            if (!f) return nullptr;
-            Group& g = groups[std::make_pair(f, cp.C ? 16 + cp.C : (int)big)];
+            const void* f = cp.C ? cp.fn : q.fn;
+            if (!f) {
+                set_error("no kernel for this PSF size");
+                return MIRAGE_ERR_UNSUPPORTED;
+            }
+            Group*& gp = cl.group[k];
+            if (k > 0 && cl.form[k] == cl.form[k - 1])
+                gp = cl.group[k - 1];
+            else
+                gp = &groups[std::make_pair(f, cp.C ? 16 + cp.C : (int)q.big)];
+            Group& g = *gp;
             g.fn = f;
-            g.big = big;
-            g.fast = fast;
+            g.fast = q.fast;
             g.cl = cp.C;
             g.nt = cp.C ? cp.nt : NTHREADS;
-            g.prob = (g.prob == -1 || g.prob == prob_idx[c]) ? prob_idx[c] : -2;
-            g.per_sm = per_sm;
-            g.smem = std::max(g.smem, cp.C ? cp.smem : item_smem);
-            g.slab = std::max<long long>(g.slab, cp.C ? cp.slab : item_slab);
-            g.load += form.it.lat * chain_weight(n_lam[c], k);
-            g.longest = std::max(g.longest, form.it.lat * w);
-            ++ctx->last_kernels[cp.C ? 3 + (cp.C > 1) + (cp.C > 2) + (cp.C > 4) : fast ? 0 : P.fft_m ? 2 : 1];
-            return &g;
-        };
-        for (int k = n_lam[c] - 1; k > 0; --k)
-            if (lam_start) group_of(k);
-        Group* g0 = group_of(0);
-        if (!g0) {
-            set_error("no kernel for this PSF size");
-            return MIRAGE_ERR_UNSUPPORTED;
+            g.prob = (g.prob == -1 || g.prob == cl.p) ? cl.p : -2;
+            g.per_sm = q.per_sm;
+            g.smem = std::max(g.smem, cp.C ? cp.smem : q.smem);
+            g.slab = std::max<long long>(g.slab, cp.C ? cp.slab : q.slab);
+            g.load += cl.count * form.it.lat * w[k];
+            g.longest = std::max(g.longest, form.it.lat * w[k]);
+            ctx->last_kernels[cp.C ? 3 + (cp.C > 1) + (cp.C > 2) + (cp.C > 4) : q.fast ? 0 : hp[cl.p].fft_m ? 2 : 1] += cl.count;
         }
-        Group& g = *g0;
+    }
+    // chained calls: each CTA slot's share of the estimated cost of the call
+    double chain_budget = 0.0;
+    if (lam_start) {
+        double tw = 0.0;
+        for (auto& kv : classes) {
+            const Prob<T>& P = hp[kv.second.p];
+            const double work = (double)P.plen * P.K * P.K + 8.0 * P.nrays;
+            for (double wk : weight[kv.second.n]) tw += kv.second.count * work * wk;
+        }
+        chain_budget = tw / (double)cgls_slots(ctx, 2);
+    }
+    for (int c = 0; c < n_cand; ++c) {
+        const Prob<T>& P = hp[prob_idx[c]];
+        const std::vector<Group*>& group = class_of[c]->group;
         const double work = (double)P.plen * P.K * P.K + 8.0 * P.nrays;
         // lambda grids ascend: smaller k = smaller lambda = more CG iterations
         auto cost_of = [&](int k) { return work * (double)(n_lam[c] - k + 4); };
@@ -989,9 +1035,10 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
             // iteration counts of log-spaced grids, which grow geometrically
             // towards small lambda
             const int ks = std::min(std::max(lam_start[c], 0), n_lam[c] - 1);
-            auto wk = [&](int k) { return work * chain_weight(n_lam[c], k); };
+            const std::vector<double>& w = weight[n_lam[c]];
+            auto wk = [&](int k) { return work * w[k]; };
             auto push_run = [&](int ka, int kb, double cd) {
-                g.items.push_back({-cd, pack_chain(c, ka, kb)});
+                group[0]->items.push_back({-cd, pack_chain(c, ka, kb)});
             };
             int ka = ks;
             double cd = 0.0;
@@ -1018,7 +1065,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                 push_run(ka, n_lam[c] - 1, cd);
             }
         } else {
-            for (int k = 0; k < n_lam[c]; ++k) (k ? group_of(k) : g0)->items.push_back({-cost_of(k), pack_chain(c, k, k)});
+            for (int k = 0; k < n_lam[c]; ++k) group[k]->items.push_back({-cost_of(k), pack_chain(c, k, k)});
         }
     }
     std::vector<int> all_items;
@@ -1308,20 +1355,10 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
             }
             for (int c = 0; c < n_cand && !rc; ++c) {
                 const Prob<T>& P = hp[prob_idx[c]];
-                const int place = pick_place<T>(ctx, P, o.place);
-                const void* fn = pick_cgls(prec, place, P.fft_m ? 0 : P.K);
-                size_t item_smem = smem_bytes<T>(P, layout_of(place));
-                int pmode = 0;
-                bool pfast = false;
-                if (const void* ff = choose(P, pmode, pfast)) {
-                    fn = ff;
-                    item_smem = fast_smem_bytes(*reinterpret_cast<const Prob<float>*>(&P));
-                }
-                const ClusterPlan& cp = form_of(prob_idx[c], 1.0, limit).cp;
-                if (cp.C) {
-                    fn = cp.fn;
-                    item_smem = cp.smem;
-                }
+                const ProbPlan& q = plan[prob_idx[c]];
+                const ClusterPlan& cp = class_of[c]->form[0]->cp;
+                const void* fn = cp.C ? cp.fn : q.fn;
+                const size_t item_smem = cp.C ? cp.smem : q.smem;
                 TRY(set_smem(ctx, fn, item_smem));
                 int cand0 = c, nc = 1;
                 rc = launch_raytrace<T>(ctx, dprobs, dcand, d_lens, c, 1, cs, max_cells, max_npix, max_rays, st);
@@ -1333,18 +1370,18 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                     A.max_smem = cluster_smem_limit(ctx, cp.nt);
                     void* a2[] = {&A};
                     rc = launch_cluster(ctx, fn, A.n_items, cp.C, cp.nt, a2, item_smem, st);
-                } else if (pfast) {
+                } else if (q.fast) {
                     FastArgs fa;
                     std::memset(&fa, 0, sizeof(fa));
                     set_fast_args<T>(fa, A);
-                    if (pmode > 0) {
+                    if (q.mode > 0) {
                         std::vector<T> psf((size_t)P.K * P.K);
                         CK(cudaMemcpy(psf.data(), P.psf, sizeof(T) * P.K * P.K, cudaMemcpyDefault));
                         for (int a = 0; a < P.K; ++a)
                             for (int b = 0; b < P.K; ++b) {
                                 fa.ptap[0][a * P.K + b] =
-                                    tap_value((float)psf[(P.K - 1 - a) * P.K + (P.K - 1 - b)], pmode == 3);
-                                fa.ptap[1][a * P.K + b] = tap_value((float)psf[a * P.K + b], pmode == 3);
+                                    tap_value((float)psf[(P.K - 1 - a) * P.K + (P.K - 1 - b)], q.mode == 3);
+                                fa.ptap[1][a * P.K + b] = tap_value((float)psf[a * P.K + b], q.mode == 3);
                             }
                     }
                     void* a2[] = {&fa};
