@@ -354,42 +354,77 @@ struct ClusterPlan {
     long long slab = 0;
 };
 
-// Clocks of one CG iteration of problem P: `lat` as one item sees it, `thr`
-// the SM clocks that it takes up.  Fits to measured iterations, good to about
-// 20% (one candidate, one lambda, refinement included; clocks / 1000; image,
-// source, K: general kernel with everything in shared memory, then the cluster
-// kernel on 1, 2, 4 and 8 SMs):
-//   48 48 11: 43, 90, 55, 42, 33   48 32 15: 34, 47, 33, 25, 23
-//   64 32 15: 37, 55, 34, 28, 23   96 48 11: (96), 76, 48, 38, 30
-//   128 48 15: (172), -, 99, 78, 57   256 128 21: (1555), -, -, -, 159
-// (in brackets: not all in shared memory; there the time of a loaded device
-// counts, where the slabs' traffic adds up: 2048 items at 256 x 256 and K = 21 took
-// 1155 of SM time an iteration with two CTAs an SM, and clusters of eight, of which
-// 15 fit the 152 SMs, 1611).  A source about as fine as the image
-// has its L^T summed ray by ray (`gather`), which costs both kernels clocks per
-// source pixel.  The two-CTA kernel: 27.5 each of two at 64 x 64, K = 9.
+// Clocks of one CG iteration of problem P: `lat` as one item alone sees it, `thr`
+// the SM clocks that it takes up on a busy device, `busy` as an item sees it there
+// (with another item's CTAs on its SMs where two fit).  Least-squares fits to the
+// iterations of 147 systems (images 28 x 28 to 256 x 256, sources 12 x 12 to 128 x 128,
+// K = 3 to 21, fields of 3.2 to 6.4 arcsec; one item alone, and 304 of them
+// together), which they meet to 10% (general kernel, everything in shared memory),
+// 15% (not everything) and 13% (cluster kernel).
 struct IterCost {
-    double lat, thr;
+    double lat, thr, busy;
 };
+// mapped part of the image: the source's area, magnified (measured: 0.6 to 0.95
+// where the areas' ratio is 0.19 to 0.26, 0.27 at 0.06)
+template <typename T>
+double mapped_part(const Prob<T>& P) {
+    const double area = P.hx * P.sx * P.hy * P.sy / (P.npix * P.pix * P.pix);
+    return std::min(1.0, 0.07 + 3.2 * area);
+}
+// a source about as fine as the image has its L^T summed ray by ray
+template <typename T>
+bool gathers(const Prob<T>& P) {
+    return 4 * P.ncells > P.plen;
+}
 template <typename T>
 IterCost fast_cost(const Prob<T>& P) {
-    const double c = 4.0 * P.K * P.K * P.npix / 130.0 + P.nrays;
-    return {2.0 * c, c};
+    const double c = 4.0 * P.K * P.K * P.npix / 130.0 + P.nrays;  // (27.5k each of two at 64 x 64, K = 9)
+    return {2.0 * c, c, 2.0 * c};
 }
 template <typename T>
 IterCost general_cost(const Prob<T>& P, int place) {
-    if (P.fft_m) return {6.0 * P.fft_m * P.fft_m, 6.0 * P.fft_m * P.fft_m};
-    const int per = (P.ntiles + NTHREADS - 1) / NTHREADS;
-    double c = 14500.0 + 73.0 * P.K * P.K * per + 1.5 * P.nrays + (4 * P.ncells > P.plen ? 7.2 * P.ns : 0.0);
-    if (place == PLACE_SMEM || place == PLACE_SMEM2) return {c, c};
-    c = 11.7 * P.nrays + 111.0 * P.K * P.K * per;
-    if (layout_of(place) == PLACE_MID) return {0.58 * c, 0.84 * c};
-    return {c, two_per_sm(place) ? 0.75 * c : c};
+    if (P.fft_m) return {6.0 * P.fft_m * P.fft_m, 6.0 * P.fft_m * P.fft_m, 6.0 * P.fft_m * P.fft_m};
+    // PSF widths without a kernel of their own loop over the taps at run time
+    const bool unrolled = P.K < MAX_K && table().cgls[prec_of<T>()][place][P.K];
+    const double k2 = P.K * P.K, per = (P.ntiles + NTHREADS - 1) / NTHREADS, pix = P.npix;
+    const double rays = mapped_part(P) * P.nrays, fine = gathers(P) ? P.ns : 0.0;
+    if (place == PLACE_SMEM || place == PLACE_SMEM2) {
+        const double c = unrolled ? 7000.0 + 61.0 * k2 * per + 4.6 * pix + 0.2 * rays + 7.3 * fine
+                                  : 9200.0 + k2 * (1.72 * P.ntiles + 81.0 * per) + 1.2 * pix + 3.5 * rays + 10.5 * fine;
+        return {c, 1.05 * c, 1.05 * c};
+    }
+    if (layout_of(place) == PLACE_MID) {
+        const double c = unrolled ? 78.0 * k2 * per + 4.2 * pix + 3.1 * rays + 780.0 * rays / P.ncells
+                                  : 58000.0 + k2 * (0.93 * P.ntiles + 184.0 * per) + 3.4 * rays;
+        return {c, 1.07 * c, 1.07 * c};
+    }
+    // (the slabs' traffic adds up: 2048 items at 256 x 256 and K = 21 took 1155k of SM
+    // time an iteration with two CTAs an SM)
+    const double c = (unrolled ? 123.0 : 430.0) * k2 * per + 5.9 * pix + 6.6 * rays;
+    return {c, two_per_sm(place) ? 0.8 * c : c, two_per_sm(place) ? 1.6 * c : c};
 }
 inline IterCost cluster_cost(const Prob<float>& P, int C, int nt) {
-    const double conv = 4.0 * P.K * P.K * P.npix, rays = P.nrays;
-    const double lat = 20000.0 + 0.6 * rays + (conv / 170.0 + 3.5 * rays + (4 * P.ncells > P.plen ? 25.0 * P.ns : 0.0)) / C;
-    return {lat, lat * C * (nt > NTHREADS ? 1.0 : 0.85) * (C == 8 ? 1.27 : 1.0)};
+    // a cell's rays are one thread's; of coarse sources, whole rows of cells are one
+    // CTA's (13 x 14 cells on eight SMs: 164k clocks)
+    const double f = mapped_part(P), rays = f * P.nrays, conv = f * P.K * P.K * P.npix, pix = P.npix;
+    const double cell = rays / P.ncells, crowd = std::max(0.0, cell - 30.0), fine = gathers(P) ? P.ns : 0.0;
+    const double lat = 18200.0 + 0.75 * rays + 700.0 * cell + 1000.0 * std::min(C, 4) * crowd +
+                       (4000.0 + 2.6 * rays + 0.0185 * conv + 0.3 * pix + 20.4 * fine) / C;
+    // SM time by CTA (two of 256 threads an SM, or one of 512) and cluster size: the
+    // barriers' waits are partly the other CTA's, and no whole cluster fits on some SMs
+    // (15 of eight on 152).  {1, rays, conv, pix, cell, crowd, fine}; the last two
+    // of 512 threads from two image sizes
+    static constexpr double w[2][4][7] = {{{11100, 2.38, 0.0144, 2.28, 461, 0, 11.4},
+                                           {23400, 2.29, 0.0158, 1.05, 872, 2500, 11.7},
+                                           {49400, 3.27, 0.0218, 1.54, 1730, 13100, 16.5},
+                                           {86400, 5.87, 0.0203, 1.30, 3300, 33200, 23.1}},
+                                          {{15600, 1.98, 0.0126, 2.58, 913, 1000, 0},
+                                           {41400, 4.98, 0.0157, 1.15, 984, 2700, 0},
+                                           {86000, 6.30, 0.0360, 1.00, 1730, 13100, 0},
+                                           {90000, 14.9, 0.0218, 3.90, 3300, 33200, 0}}};
+    const double* a = w[nt > NTHREADS][(C > 1) + (C > 2) + (C > 4)];
+    const double thr = a[0] + a[1] * rays + a[2] * conv + a[3] * pix + a[4] * cell + a[5] * crowd + a[6] * fine;
+    return {lat, thr, nt > NTHREADS ? lat : std::max(lat, 2.0 * thr / C)};
 }
 
 // dynamic shared memory of a cluster-kernel CTA: two CTAs of 256 threads share
@@ -824,22 +859,21 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         return f;
     };
     // Kernel of the items that the two-CTA kernel does not take, unless a kernel
-    // or a placement of the general kernel is asked for.  A problem has up to two
-    // forms: the one that takes the least SM time an iteration (the general kernel
-    // where everything fits in shared memory, or the cluster kernel of some size),
-    // and the one with the shortest iteration.  Items that would outlast the call
-    // in the first form take the second.  All forms give the same bits.  (48 x 48
-    // image and source, K = 15, one item: 23.7 us an iteration in the general
-    // kernel, 13.8 on a cluster of eight SMs; 304 such items 25 ms in the general
-    // kernel and 33 on clusters of four)
+    // or a placement of the general kernel is asked for: the general kernel, or the
+    // cluster kernel on 1, 2, 4 or 8 SMs.  All forms give the same bits.  (48 x 48 image
+    // and source, K = 15: one item takes 23.7 us an iteration in the general kernel and
+    // 13.8 on eight SMs; 304 such items 25 ms in the general kernel and 33 on
+    // clusters of four)
     struct Form {
         IterCost it;
         ClusterPlan cp;  // C = 0: general or two-CTA kernel
     };
     // what a problem's items have in common
     struct ProbPlan {
-        Form cheap, quick;
-        bool whole = false;  // one form for all items
+        std::vector<Form> forms;  // [0]: without clusters; all by SM time an iteration, least first, in order
+        std::vector<int> order;
+        int quick = 0;            // the form with the shortest iteration
+        double iters = 1.0;       // iterations of an item, relative to other problems'
         const void* fn = nullptr;  // the kernel without clusters, its shared memory, slab, CTAs per SM
         size_t smem = 0;
         long long slab = 0;
@@ -847,7 +881,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         bool fast = false, big = false;
     };
     std::vector<ProbPlan> plan(n_probs);
-    bool second = false;  // some problem has a second form
+    bool choice = false;  // some problem has several forms
     for (int p = 0; p < n_probs; ++p) {
         if (!cands_of[p]) continue;
         const Prob<T>& P = hp[p];
@@ -871,29 +905,25 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
             q.slab = (long long)fast_slab_bytes(*reinterpret_cast<const Prob<float>*>(&P));
             q.per_sm = 2;
         }
-        q.cheap.it = q.fast ? fast_cost(P) : general_cost(P, pick_place<T>(ctx, P, o.place));
-        q.quick = q.cheap;
+        q.forms.push_back(Form{q.fast ? fast_cost(P) : general_cost(P, place), ClusterPlan()});
         if constexpr (sizeof(T) == 4) {
-            if (q.fast || o.place != 0 || want == 4 || want == 5 || want == 6) continue;
-            const bool in_smem = pick_place<T>(ctx, P) == PLACE_SMEM;
-            bool any = in_smem;
-            for (int C = 1; C <= CL_MAX; C *= 2) {
-                Form x;
-                if (!cluster_fits<T>(ctx, P, C, x.cp)) continue;
-                x.it = cluster_cost(P, C, x.cp.nt);
-                if (!any || x.it.thr < q.cheap.it.thr) q.cheap = x;
-                if (!any || x.it.lat < q.quick.it.lat) q.quick = x;
-                any = true;
-            }
-            // the general kernel on its slabs where its work a device is less; all
-            // items of the problem or none, since its CTAs would hold up clusters
-            const IterCost g = general_cost(P, pick_place<T>(ctx, P));
-            if (any && !in_smem && g.thr < q.cheap.it.thr) {
-                q.cheap = Form{g, ClusterPlan()};
-                q.whole = true;
-            }
+            if (!q.fast && o.place == 0 && want != 4 && want != 5 && want != 6)
+                for (int C = 1; C <= CL_MAX; C *= 2) {
+                    Form x;
+                    if (!cluster_fits<T>(ctx, P, C, x.cp)) continue;
+                    x.it = cluster_cost(P, C, x.cp.nt);
+                    q.forms.push_back(x);
+                }
         }
-        second |= q.quick.it.lat < 0.8 * q.cheap.it.lat;
+        for (int i = 0; i < (int)q.forms.size(); ++i) {
+            q.order.push_back(i);
+            if (q.forms[i].it.lat < q.forms[q.quick].it.lat) q.quick = i;
+        }
+        std::stable_sort(q.order.begin(), q.order.end(), [&](int a, int b) { return q.forms[a].it.thr < q.forms[b].it.thr; });
+        choice |= q.forms.size() > 1;
+        // (25 to 36 at K = 3, 110 at 9, 170 at 15, 360 to 560 at 21, for PSFs of K / 6
+        // pixels at one lambda; sources of 256 and 2304 pixels: 1 to 1.4)
+        q.iters = P.K * std::pow((double)P.ns, 0.15);
     }
     // candidates of one problem and lambda count are alike: their items' forms and
     // groups are looked up once, and the weights of an n-point grid made once
@@ -906,6 +936,11 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     std::map<std::pair<int, int>, Class> classes;
     std::vector<Class*> class_of(n_cand);
     std::vector<std::vector<double>> weight(max_lam + 1);
+    // iteration counts for estimates, by how they may fall from the smallest lambda
+    // to the largest (see estimate)
+    constexpr double FALL[2] = {0.8, 2.0};
+    std::vector<std::vector<double>> fall[2];
+    for (auto& f : fall) f.resize(max_lam + 1);
     for (int c = 0; c < n_cand; ++c) {
         Class*& cl = class_of[c];
         if (c > 0 && prob_idx[c] == prob_idx[c - 1] && n_lam[c] == n_lam[c - 1]) {
@@ -916,65 +951,107 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
             cl->n = n_lam[c];
         }
         cl->count++;
-        std::vector<double>& w = weight[n_lam[c]];
-        for (int k = (int)w.size(); k < n_lam[c]; ++k) w.push_back(chain_weight(n_lam[c], k));
-    }
-    // form of an item of problem p with w iterations where items may take `limit` clocks
-    auto form_of = [&](const ProbPlan& q, double w, double limit) -> const Form& {
-        return w * q.cheap.it.lat > limit && q.quick.it.lat < 0.8 * q.cheap.it.lat ? q.quick : q.cheap;
-    };
-    auto set_forms = [&](double limit) {
-        for (auto& kv : classes) {
-            Class& cl = kv.second;
-            const ProbPlan& q = plan[cl.p];
-            const std::vector<double>& w = weight[cl.n];
-            cl.form.resize(cl.n);
-            for (int k = 0; k < cl.n; ++k)
-                cl.form[k] = &form_of(q, w[lam_start && o.mode == MIRAGE_MODE_BATCHED ? 0 : k], limit);
-            if (q.whole) std::fill(cl.form.begin(), cl.form.end(), cl.form[0]);
+        const int n = n_lam[c];
+        for (int k = (int)weight[n].size(); k < n; ++k) {
+            weight[n].push_back(chain_weight(n, k));
+            for (int j = 0; j < 2; ++j)
+                fall[j][n].push_back(chain_weight(n, 0) * std::pow(10.0, -FALL[j] * k / std::max(1, n - 1)));
         }
+    }
+    // forms of some classes' items where an item may take `limit` clocks: the one of
+    // least SM time that takes no longer, or else the quickest.  Without `each`, one
+    // form for all items of a class (that of the smallest lambda's); limit < 0: no
+    // clusters.  False once a larger limit changes nothing more
+    typedef std::vector<Class*> Classes;
+    const bool chains = lam_start && o.mode == MIRAGE_MODE_BATCHED;
+    auto set_forms = [&](const Classes& some, double limit, bool each) {
+        bool more = false;
+        for (Class* cl : some) {
+            const ProbPlan& q = plan[cl->p];
+            cl->form.resize(cl->n);
+            for (int k = 0; k < cl->n; ++k) {
+                if (k > 0 && !each) {
+                    cl->form[k] = cl->form[0];
+                    continue;
+                }
+                const double w = q.iters * weight[cl->n][k];
+                int f = limit < 0.0 ? 0 : q.quick;
+                if (limit >= 0.0)
+                    for (int i : q.order)
+                        if (w * q.forms[i].it.lat <= limit) {
+                            f = i;
+                            break;
+                        }
+                more |= f != q.order[0];
+                cl->form[k] = &q.forms[f];
+            }
+        }
+        return more;
     };
-    double call_time = 0.0;  // estimated clocks of the call
-    set_forms(o.mode == MIRAGE_MODE_PLAIN ? 0.0 : 1e300);  // (plain mode: one candidate at a time)
-    if (second && o.mode == MIRAGE_MODE_BATCHED) {
-        // the call's time as a function of the limit: its longest item, or its work
-        // on all SMs, and part of the other one (the end of a call is never packed
-        // full)
-        double total = 0.0, best = 1e300, limit = 1e300;
-        for (auto& kv : classes)
-            for (double wk : weight[kv.second.n]) total += kv.second.count * wk * plan[kv.second.p].cheap.it.thr / ctx->sm_count;
-        for (double T_ = 0.5 * total; T_ < 1e3 * total; T_ *= 1.5) {
-            set_forms(T_);
-            double sum = 0.0, longest = 0.0;
-            bool other = false;  // items in their second form
-            for (auto& kv : classes) {
-                const Class& cl = kv.second;
-                const std::vector<double>& w = weight[cl.n];
-                for (int k = 0; k < cl.n; ++k) {
-                    sum += cl.count * w[k] * cl.form[k]->it.thr / ctx->sm_count;
-                    longest = std::max(longest, w[k] * cl.form[k]->it.lat);
-                    other |= !plan[cl.p].whole && cl.form[k] == &plan[cl.p].quick;
+    // Estimated clocks of the classes' items with these forms: the longest item (1.15
+    // of the mean over candidates, up to 2 where problems differ), or the work on all SMs, and
+    // part of the other one, since the end of a call is never packed full.  How iteration
+    // counts fall with lambda depends on the grid's values, which are device data: the
+    // estimate is the geometric mean over counts that fall by 10^0.8 and by 10^2 from
+    // the smallest lambda to the largest.  (Against the general kernel alone: 120 drawn
+    // calls of 28 to 100 pixels a side and 1 to 128 candidates 1.40 times as fast in the
+    // mean, the slowest 0.85; 14 calls of 12 to 400 unlike problems 1.3 to 4.1 times.)
+    const double unlike = std::min(1.0, 0.125 * (n_used - 1));  // nine problems and more: 1
+    double call_time = 0.0;                                     // (with the second)
+    auto estimate = [&](const Classes& some, bool together) {
+        double e = 0.0;
+        bool cluster = false;
+        for (const auto& ws : fall) {
+            double sum = 0.0, alone = 0.0, busy = 0.0;
+            for (const Class* cl : some) {
+                const double it = plan[cl->p].iters;
+                for (int k = 0; k < cl->n; ++k) {
+                    const double w = it * ws[cl->n][k];
+                    sum += (together ? cl->count : 1) * w * cl->form[k]->it.thr / ctx->sm_count;
+                    alone = std::max(alone, w * cl->form[k]->it.lat);
+                    busy = std::max(busy, w * cl->form[k]->it.busy);
+                    cluster |= cl->form[k]->cp.C > 0 && !plan[cl->p].big;
                 }
             }
-            const double est = std::max(sum, longest) + 0.5 * std::min(sum, longest);
-            if (est < 0.98 * best) {
-                best = est;
-                limit = T_;
-                call_time = std::max(sum, longest);
-            }
-            if (!other) break;  // every item in the first form: a larger limit changes nothing more
+            const double full = 0.5 * std::min(1.0, sum / busy);  // its part beside others
+            const double longest = ((1.0 - full) * alone + full * busy) * (1.15 + 0.85 * unlike);
+            e += 0.5 * std::log(std::max(sum, longest) + 0.3 * std::min(sum, longest));
+            call_time = std::max(sum, longest);
         }
-        set_forms(limit);
-    } else if (plan.size() > 1) {
-        double sum = 0.0, longest = 0.0;
-        for (auto& kv : classes)
-            for (int k = 0; k < kv.second.n; ++k) {
-                const IterCost& it = kv.second.form[k]->it;
-                sum += kv.second.count * weight[kv.second.n][k] * it.thr / ctx->sm_count;
-                longest = std::max(longest, weight[kv.second.n][k] * it.lat);
+        // clusters in place of the general kernel with everything in shared memory have to
+        // be better by 1.1
+        return e + (cluster ? 0.1 : 0.0);
+    };
+    auto search = [&](const Classes& some, bool together, bool mixed) {
+        set_forms(some, -1.0, false);
+        double best = estimate(some, together), limit = -1.0;
+        const double first = call_time;
+        bool each = false;
+        for (int m = 0; m <= (int)mixed; ++m)
+            for (double T_ = 0.0, more = 1.0; more; T_ = std::max(1.5 * T_, 0.1 * first)) {
+                more = set_forms(some, T_, m == 1);
+                // a plan that mixes the forms of one problem has to be better by 1.02 (forms
+                // in turn hold each other up); with many unlike problems and few items a SM
+                // it may be worse by 1.05
+                const double e = estimate(some, together) + (n_items < 8LL * ctx->sm_count ? 0.02 - 0.07 * unlike : 0.02) * m;
+                if (e < best) {
+                    best = e;
+                    limit = T_;
+                    each = m == 1;
+                }
             }
-        call_time = std::max(sum, longest);
+        set_forms(some, limit, each);
+    };
+    Classes all;
+    for (auto& kv : classes) all.push_back(&kv.second);
+    if (!choice) {
+        set_forms(all, -1.0, false);
+    } else if (o.mode == MIRAGE_MODE_PLAIN) {  // one candidate at a time
+        for (Class* cl : all) search(Classes(1, cl), false, false);
+    } else {
+        search(all, true, !chains);  // (a chain's items share a kernel)
     }
+    if (all.size() > 1 || choice) estimate(all, true);
     // groups: items of one kernel (and cluster size) share a launch
     std::fill(ctx->last_kernels, ctx->last_kernels + MIRAGE_N_ITEM_KERNELS, 0);
     for (auto& kv : classes) {
@@ -1004,8 +1081,8 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
             g.per_sm = q.per_sm;
             g.smem = std::max(g.smem, cp.C ? cp.smem : q.smem);
             g.slab = std::max<long long>(g.slab, cp.C ? cp.slab : q.slab);
-            g.load += cl.count * form.it.lat * w[k];
-            g.longest = std::max(g.longest, form.it.lat * w[k]);
+            g.load += cl.count * q.iters * w[k] * form.it.lat;
+            g.longest = std::max(g.longest, q.iters * w[k] * form.it.lat);
             ctx->last_kernels[cp.C ? 3 + (cp.C > 1) + (cp.C > 2) + (cp.C > 4) : q.fast ? 0 : hp[cl.p].fft_m ? 2 : 1] += cl.count;
         }
     }

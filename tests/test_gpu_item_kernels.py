@@ -8,7 +8,7 @@ import torch
 
 import synth
 
-from .test_gpu_cluster import L, _problem
+from .test_gpu_cluster import G, I, L, _problem
 
 pytestmark = pytest.mark.gpu
 
@@ -48,3 +48,38 @@ def test_options_that_name_a_kernel():
     assert _kernels([f], 2, 3)["two_cta"] == 6
     assert _kernels([f, (48, 48, 24, 24, 33)], 4, 3)["fft"] == 6
     assert _kernels([f], 2, 3, use_graph=True)["two_cta"] == 6
+
+
+KEYS = ("chi2", "reg", "iters", "relres", "item_status", "corner", "status", "kappa", "all_x")
+
+
+@pytest.mark.parametrize("shape,n,ran", [
+    ((64, 64, 32, 32, 15, L), 12, ["cluster1", "cluster8"]),     # CTAs of 256 threads
+    ((60, 44, 24, 27, 13, G), 100, ["cluster1"]),
+    ((48, 40, 33, 31, 3, I), 12, ["cluster1", "cluster8"]),      # L^T ray by ray
+    ((100, 100, 36, 36, 9, L), 100, ["cluster1"]),               # CTAs of 512
+    ((72, 72, 36, 36, 13, L), 100, ["cluster2"]),
+    ((64, 64, 60, 62, 21, L), 100, ["cluster2"]),                # ray by ray, more rays than are staged
+    ((131, 45, 17, 19, 5, I), 40, ["cluster2"]),
+    ((128, 128, 48, 48, 11, L), 200, ["cluster2"]),              # 512
+    ((128, 128, 48, 48, 11, L), 40, ["cluster4"]),
+    ((32, 32, 16, 16, 13, L), 1, ["cluster4"]),
+    ((200, 200, 96, 96, 15, L), 40, ["cluster4"]),               # 512
+    ((97, 83, 31, 40, 7, G), 1, ["cluster8"]),
+    ((200, 200, 96, 96, 15, L), 4, ["cluster8"]),                # 512
+])
+def test_every_cluster_size_gives_the_general_kernels_bits(shape, n, ran):
+    from paper_1101_5803_gb300 import binding
+    ctx = binding.Context(0, binding.MIRAGE_FP32)
+    p = _problem(ctx, *shape, 3)
+    lens = torch.as_tensor(synth.lens_population(np.random.default_rng(7), n), device="cuda")
+    lams = torch.as_tensor(np.tile(synth.lambda_grid(3, 1.0, 1e2), (n, 1)), device="cuda")
+    run = lambda v: ctx.eval_batch([p], lens, np.zeros(n), lams, np.full(n, 3), want_all_x=True, variant=v)  # noqa: E731
+    a = run(0)
+    k = ctx.item_kernels()
+    assert all(k[r] for r in ran) and sum(k[r] for r in ran) == 3 * n, k
+    b = run(4)
+    assert ctx.item_kernels()["direct"] == 3 * n
+    for key in KEYS:
+        assert torch.equal(a[key], b[key]), key
+    ctx.close()
