@@ -56,7 +56,8 @@ KEYS = ("chi2", "reg", "iters", "relres", "item_status", "corner", "status", "ka
 @pytest.mark.parametrize("shape,n,ran", [
     ((64, 64, 32, 32, 15, L), 12, ["cluster1", "cluster8"]),     # CTAs of 256 threads
     ((60, 44, 24, 27, 13, G), 100, ["cluster1"]),
-    ((48, 40, 33, 31, 3, I), 12, ["cluster1", "cluster8"]),      # L^T ray by ray
+    ((48, 40, 33, 31, 3, I), 4, ["cluster8"]),                   # L^T ray by ray
+    ((64, 64, 60, 62, 21, L), 200, ["cluster1", "cluster2"]),
     ((100, 100, 36, 36, 9, L), 100, ["cluster1"]),               # CTAs of 512
     ((72, 72, 36, 36, 13, L), 100, ["cluster2"]),
     ((64, 64, 60, 62, 21, L), 100, ["cluster2"]),                # ray by ray, more rays than are staged
