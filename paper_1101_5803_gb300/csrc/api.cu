@@ -1149,8 +1149,14 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
     std::vector<size_t> g_off;
     std::vector<Group*> glist;
     for (auto& kv : groups) glist.push_back(&kv.second);
-    // the group with the longest item first: the others fill in behind its tail
-    std::stable_sort(glist.begin(), glist.end(), [](const Group* a, const Group* b) { return a->longest > b->longest; });
+    // the others fill in behind the first group's tail: where the groups share the device
+    // (see the launches), first the group with the longest item, otherwise the one
+    // with the most work
+    bool shared = n_items < 4LL * ctx->sm_count;
+    for (Group* g : glist) shared |= g->cl > 0;
+    std::stable_sort(glist.begin(), glist.end(), [&](const Group* a, const Group* b) {
+        return shared ? a->longest > b->longest : a->load > b->load;
+    });
     for (Group* gp : glist) {
         Group& g = *gp;
         std::stable_sort(g.items.begin(), g.items.end(),
@@ -1364,20 +1370,25 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                 cudaEventRecord(ctx->fork_ev, st);
                 for (int i = 0; i < n_side; ++i) cudaStreamWaitEvent(ctx->side[i], ctx->fork_ev, 0);
             }
-            // Several groups share the device from the start, each with the CTAs that
-            // finish its items in the call's estimated time (and half as many more:
-            // iteration counts are estimates), and each launches the rest of the CTAs
-            // that it could use behind them: those start as other groups end.  (One
-            // group after the other, each on all SMs, leaves the last group's longest
-            // item alone on the device: the uneven batch of 48 candidates then ran at
-            // 0.97 of the speed of the general kernels alone, side by side at 1.40.)
-            for (int part = 0; part < (fork ? 2 : 1) && !rc; ++part)
+            // Groups share the device from the start where there are clusters or few items
+            // a SM, each with the CTAs that finish its items in the call's estimated time
+            // (and half as many more: iteration counts are estimates), and each launches
+            // the rest of the CTAs that it could use behind them: those start as other
+            // groups end.  (One group after the other, each on all SMs, leaves the last
+            // group's longest item alone on the device: the uneven batch of 48 candidates
+            // then ran at 0.97 of the speed of the general kernels alone, side by side at
+            // 1.40; two PSF widths at 64 x 64, 32 candidates x 12 lambdas, 13.1 and 10.2 ms.)
+            // Many items fill in behind each other anyway, and shares cost more than they
+            // give: four PSF widths, 192 candidates, 27.2 ms one after the other, 28.5 to
+            // 31 side by side
+            const bool split = fork && shared;
+            for (int part = 0; part < (split ? 2 : 1) && !rc; ++part)
                 for (size_t gi = 0; gi < glist.size() && !rc; ++gi) {
                     Group* g = glist[gi];
                     const cudaStream_t gs = fork ? ctx->side[(2 * gi + part) % ctx->NSIDE] : st;
                     const long long full = std::min<long long>(g->slots, (long long)g->items.size());
                     const long long first =
-                        fork ? std::min(full, std::max<long long>(1, (long long)std::ceil(1.5 * g->load / call_time))) : full;
+                        split ? std::min(full, std::max<long long>(1, (long long)std::ceil(1.5 * g->load / call_time))) : full;
                     const int grid = (int)(part == 0 ? first : full - first);
                     if (!grid) continue;
                     A.slab = ctx->slab.as<unsigned char>() + (g_slab_off[gi] + (part ? first : 0)) * slab_stride;

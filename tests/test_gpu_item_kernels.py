@@ -84,3 +84,25 @@ def test_every_cluster_size_gives_the_general_kernels_bits(shape, n, ran):
     for key in KEYS:
         assert torch.equal(a[key], b[key]), key
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [8, 80])
+def test_groups_side_by_side_or_in_turn(n):
+    # four PSF widths of the two-CTA kernel in one call: with few items their
+    # launches share the device (two a group), with many each takes all of it
+    from paper_1101_5803_gb300 import binding
+    ctx = binding.Context(0, binding.MIRAGE_FP32)
+    probs = [_problem(ctx, 64, 64, 32, 32, k, L, k) for k in (5, 7, 9, 11)]
+    lens = torch.as_tensor(synth.lens_population(np.random.default_rng(7), n), device="cuda")
+    lams = torch.as_tensor(np.tile(synth.lambda_grid(12, 1.0, 1e2), (n, 1)), device="cuda")
+    idx, nl = np.arange(n) % 4, np.full(n, 12)
+    a = ctx.eval_batch(probs, lens, idx, lams, nl, want_all_x=True)
+    launches = ctx.launches()
+    assert ctx.item_kernels()["two_cta"] == 12 * n
+    assert launches > 7 if n == 8 else launches == 2 + 4 + 1
+    for i in range(4):  # each problem in a call of its own
+        one = ctx.eval_batch([probs[i]], lens[i::4].contiguous(), [0] * (n // 4), lams[i::4].contiguous(), nl[i::4],
+                             want_all_x=True, variant=1)
+        for key in KEYS:
+            assert torch.equal(a[key][i::4], one[key]), key
+    ctx.close()
