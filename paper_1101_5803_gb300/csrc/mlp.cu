@@ -10,6 +10,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -468,11 +469,10 @@ struct mirage_mlp {
     int step = 0;
     float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     Buf P, PH, M, V, G, ISW;   // params FP32, BF16 copy, Adam m, v, grads, weight mask
-    Buf Z, A, DZ, DZH, DA, LOSS;  // per-batch work (grown on demand; DZ and DZH twice: a layer's and the next one's)
-    Buf IDX, DSTEP;            // device-side training loop: minibatch rows, step counter
+    Buf Z, A, DZ, DZH, LOSS;   // per-batch work (grown on demand; DZ and DZH twice: a layer's and the next one's)
+    Buf IDX, DSTEP, Y;         // device-side training loop: minibatch rows, step counter, output
     cudaStream_t cap = nullptr;  // private stream on which the training step is captured
-    long cap_rows = 0;
-    int maxw = 0;              // widest layer
+    long cap_rows = 0, cap_grad = 0;  // rows that A holds, and the gradients' buffers
     std::vector<long> z_off, a_off;  // per layer offsets into Z / A (elements)
 };
 
@@ -485,34 +485,46 @@ constexpr int layer_smem() {
     return tc_smem_bytes<BN>() > 256 * 32 * 4 ? tc_smem_bytes<BN>() : 256 * 32 * 4;
 }
 
-int ensure_batch(mirage_mlp* m, int n) {
+// Work space for passes on n rows: activations alone for a prediction, and for a
+// gradient the pre-activations and two layers' gradients as well.  A buffer that
+// fails to grow is gone, so no batch fits until all are there, and the offsets
+// change with the capacity.
+int ensure_rows(mirage_mlp* m, int n) {
     if (n <= m->cap_rows) return MIRAGE_OK;
-    long zt = 0, at = 0;
-    std::vector<long> z_off(m->L + 1, 0), a_off(m->L + 1, 0);
-    int maxw = 0;
+    std::vector<long> off(m->L + 1, 0);
+    long at = 0;
     for (int l = 0; l <= m->L; ++l) {
-        a_off[l] = at;
+        off[l] = at;
         at += ((long)n * m->dims[l] + 7) & ~7L;  // (16-byte rows stay aligned)
-        maxw = std::max(maxw, m->dims[l]);
-        if (l > 0) {
-            z_off[l] = zt;
-            zt += (long)n * m->dims[l];
-        }
     }
-    // A buffer that fails to grow is gone, and others have grown by then: no batch
-    // fits until all are there, and the offsets change with the capacity
     m->cap_rows = 0;
-    int r;
-    if ((r = m->Z.ensure(sizeof(float) * zt))) return r;
-    if ((r = m->A.ensure(sizeof(__nv_bfloat16) * at))) return r;
-    if ((r = m->DZ.ensure(2 * sizeof(float) * (((long)n * maxw + 7) & ~7L)))) return r;
-    if ((r = m->DZH.ensure(2 * sizeof(__nv_bfloat16) * (((long)n * maxw + 7) & ~7L)))) return r;
-    if ((r = m->DA.ensure(sizeof(float) * (long)n * maxw))) return r;
-    if ((r = m->LOSS.ensure(sizeof(double)))) return r;
-    m->z_off = z_off;
-    m->a_off = a_off;
-    m->maxw = maxw;
+    if (const int r = m->A.ensure(sizeof(__nv_bfloat16) * at)) return r;
+    m->a_off = off;
     m->cap_rows = n;
+    return MIRAGE_OK;
+}
+
+// elements of one layer's gradient
+long grad_rows(const mirage_mlp* m, long n) {
+    return (n * *std::max_element(m->dims.begin(), m->dims.end()) + 7) & ~7L;
+}
+
+int ensure_grad(mirage_mlp* m, int n) {
+    int r;
+    if ((r = ensure_rows(m, n))) return r;
+    if (n <= m->cap_grad) return MIRAGE_OK;
+    std::vector<long> off(m->L + 1, 0);
+    long zt = 0;
+    for (int l = 1; l <= m->L; ++l) {
+        off[l] = zt;
+        zt += (long)n * m->dims[l];
+    }
+    m->cap_grad = 0;
+    if ((r = m->Z.ensure(sizeof(float) * zt)) || (r = m->DZ.ensure(2 * sizeof(float) * grad_rows(m, n))) ||
+        (r = m->DZH.ensure(2 * sizeof(__nv_bfloat16) * grad_rows(m, n))) || (r = m->LOSS.ensure(sizeof(double))))
+        return r;
+    m->z_off = off;
+    m->cap_grad = n;
     return MIRAGE_OK;
 }
 
@@ -569,7 +581,7 @@ int launch_layer(LayerArgs& a, cudaStream_t st) {
 int forward_pass(mirage_mlp* m, const float* x, int n, float* y, cudaStream_t st, bool keep = false, const int* idx = nullptr,
                  const float* tgt = nullptr, long long* inc = nullptr) {
     int r;
-    if ((r = ensure_batch(m, n))) return r;
+    if ((r = keep ? ensure_grad(m, n) : ensure_rows(m, n))) return r;
     float* Z = (float*)m->Z.p;
     __nv_bfloat16* A = (__nv_bfloat16*)m->A.p;
     const float* P = (const float*)m->P.p;
@@ -627,7 +639,7 @@ int backward_pass(mirage_mlp* m, const float* x, const float* tgt, int n, float*
         MCK(launch_dep(k_loss_grad, blocks((long)n * outL, 256), 256, 0, st, yscratch, tgt, idx, outL, (long)n * outL,
                        (float*)m->DZ.p, (__nv_bfloat16*)m->DZH.p, loss));
     }
-    const long half = ((long)m->cap_rows * m->maxw + 7) & ~7L;  // a layer's part of DZ and DZH
+    const long half = grad_rows(m, m->cap_grad);  // a layer's part of DZ and DZH
     for (int l = m->L, cur = 0; l >= 1; --l, cur ^= 1) {
         const int in = m->dims[l - 1], out = m->dims[l];
         float *dz = (float*)m->DZ.p + cur * half, *dzn = (float*)m->DZ.p + (cur ^ 1) * half;
@@ -738,7 +750,7 @@ int mirage_mlp_destroy(mirage_mlp_t* m) {
     if (!m) return MIRAGE_OK;
     cudaSetDevice(m->device);
     Buf* bufs[] = {&m->P,  &m->PH,  &m->M,  &m->V,    &m->G,   &m->ISW,  &m->Z,
-                   &m->A,  &m->DZ,  &m->DZH, &m->DA,  &m->LOSS, &m->IDX, &m->DSTEP};
+                   &m->A,  &m->DZ,  &m->DZH, &m->Y,   &m->LOSS, &m->IDX, &m->DSTEP};
     for (Buf* b : bufs) b->release();
     if (m->cap) cudaStreamDestroy(m->cap);
     delete m;
@@ -808,13 +820,13 @@ int mirage_mlp_train(mirage_mlp_t* m, const float* x, const float* t, int n, int
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     int r;
     // every buffer the step touches exists before the capture (no allocation inside it)
-    if ((r = ensure_batch(m, batch)) || (r = m->IDX.ensure(sizeof(int) * (size_t)batch)) ||
-        (r = m->DSTEP.ensure(sizeof(long long))))
+    if ((r = ensure_grad(m, batch)) || (r = m->IDX.ensure(sizeof(int) * (size_t)batch)) ||
+        (r = m->DSTEP.ensure(sizeof(long long))) || (r = m->Y.ensure(sizeof(float) * (size_t)batch * m->dims[m->L])))
         return r;
     if (!m->cap) MCK(cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking));
     long long* dstep = (long long*)m->DSTEP.p;
     int* idx = (int*)m->IDX.p;
-    float* y = (float*)m->DA.p;  // the step's forward output (DA is free until the backward pass)
+    float* y = (float*)m->Y.p;
     const long long s0 = m->step;
     MCK(cudaMemcpyAsync(dstep, &s0, sizeof(long long), cudaMemcpyHostToDevice, st));
 
