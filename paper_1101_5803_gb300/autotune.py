@@ -23,8 +23,12 @@ probe (the placement: on the whole batch, where one evaluation of it is
 cheap).  All choices solve the same systems to the same tolerance (variants
 1-3 and the placements bitwise alike).  A shape class is the set of (image, source
 grid, PSF, sub-pixels, regulariser) of the problems, the precision and
-whether a launch mixes PSFs; its choice is cached in a JSON file and later
-calls read the cache.
+whether a launch mixes PSFs, with the batch's size to a factor of four (which
+kernel is fastest depends on the items an SM has to do: a placement that wins on
+a full device keeps a small call off the thread-block clusters, which any
+placement but 0 does); its choice is cached in a JSON file and later calls read
+the cache.  The key names the generation of the kernels as well, so that choices
+timed on others are timed again.
 """
 from __future__ import annotations
 
@@ -39,6 +43,7 @@ from .binding import MIRAGE_FP32
 VARIANTS = (0, 1, 2, 3, 4)  # 0: the library's automatic choice
 ETAS = (0.01, 0.03, 0.1)     # the first is the library's default
 PLACES = (1, 2, 3, 4, 5)
+KERNELS = 2                  # raised when kernels or their automatic choice change
 MARGIN = 0.03                # a choice must beat the default by this much to replace it
 MARGIN_PLACE = 0.05          # (a placement only moves the problems on the general kernel)
 FULL_BATCH_MS = 5000.0       # placements are re-timed on whole batches up to this cost
@@ -51,10 +56,11 @@ def cache_path() -> str:
     return os.path.join(os.path.expanduser("~"), ".cache", "mirage_gb300", "tune.json")
 
 
-def shape_key(ctx, probs) -> str:
+def shape_key(ctx, probs, n_items) -> str:
     gs = sorted({(int(p.geom.nx), int(p.geom.ny), int(p.geom.sx), int(p.geom.sy), int(p.geom.kpsf),
                   int(getattr(p.geom, "subpix", 1)), int(p.geom.reg)) for p in probs})
-    return json.dumps({"prec": int(ctx.precision), "shapes": gs, "multi": len(probs) > 1})
+    return json.dumps({"prec": int(ctx.precision), "shapes": gs, "multi": len(probs) > 1, "kernels": KERNELS,
+                       "items": max(0, int(n_items).bit_length() - 1) // 2})
 
 
 def _load():
@@ -105,7 +111,7 @@ def tune_config(ctx, probs, lens, prob_idx, lambdas, n_lam, *, tol=1e-6, n_probe
     ``full_batch_ms`` (default FULL_BATCH_MS; 0: never)."""
     if full_batch_ms is None:
         full_batch_ms = FULL_BATCH_MS
-    key = shape_key(ctx, probs)
+    key = shape_key(ctx, probs, np.sum(n_lam))
     db = _load()
     if key in db and not retune and "inner_eta" in db[key]:
         e = db[key]
