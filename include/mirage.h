@@ -129,7 +129,13 @@ typedef struct {
                           tensor-core B/B^T; 9x9 PSFs, one PSF per call; an
                           experiment on the inner solves' precision, the
                           refinement's residual stays exact).  Automatic
-                          choice: FFT for PSFs of 23 x 23 and wider, direct below.
+                          choice: FFT for PSFs of 23 x 23 and wider, direct below;
+                          FP32 problems with one ray per pixel, four-corner
+                          interpolation and K = 3..21 that the two-CTA kernel does
+                          not take run on the general kernel or on thread-block
+                          clusters of 1, 2, 4 or 8 SMs an item, by estimated time
+                          (the same bits; see mirage_last_item_kernels).  4, 5 and 6
+                          exclude the clusters.
                           Forced choices fall back to the general kernel where
                           they do not apply.  Other values: MIRAGE_ERR_ARG. */
     double inner_eta;  /* FP32 contexts: the relative residual reduction each inner
@@ -139,8 +145,11 @@ typedef struct {
                           MIRAGE_ERR_ARG.  Changes the iteration path, not the
                           solution (to tol).  FP64 contexts ignore it. */
     int place;         /* work-buffer placement of the general kernel: 0 = automatic
-                          (the most on-chip placement that fits; all in the slab
-                          means 4 where that kernel is compiled for the PSF width),
+                          (the most on-chip placement that fits, all in the slab
+                          meaning 4 where that kernel is compiled for the PSF width;
+                          or the cluster kernel, which keeps an item in several SMs'
+                          shared memory).  Any other value keeps the call off the
+                          cluster kernel:
                           1 = all in shared
                           memory, 2 = convolution inputs and source vectors in
                           shared memory, the rest in an L2-resident slab, 3 = all in

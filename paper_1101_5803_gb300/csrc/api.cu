@@ -568,9 +568,10 @@ int upload(mirage_ctx* ctx, cudaStream_t st, std::initializer_list<UploadPart> p
     return MIRAGE_OK;
 }
 
-// ray trace of candidates [cand0, cand0 + n_cand): one CTA per candidate,
-// or, for fewer candidates than SMs on large images, the split trace (many
-// CTAs per candidate trace and count, one CTA per candidate places)
+// ray trace of candidates [cand0, cand0 + n_cand): many CTAs trace and one per
+// candidate places the rays where their numbers fit in shared memory; larger
+// images: one CTA per candidate, or, for fewer candidates than SMs, the split
+// trace (many CTAs per candidate trace and count, one per candidate places)
 template <typename T>
 int launch_raytrace(mirage_ctx* ctx, const Prob<T>* dprobs, const int* dcand, const double* d_lens, int cand0,
                     int n_cand, const CandScratch<T>& cs, long long max_cells, long long max_npix, long long max_rays, cudaStream_t st);
@@ -608,8 +609,9 @@ int launch_raytrace(mirage_ctx* ctx, const Prob<T>* dprobs, const int* dcand, co
     const size_t cells_smem = (size_t)max_cells * 4;
     // Ray numbers in shared memory: two launches (one 64 x 64 candidate: 15 + 35 us;
     // a whole forward call on it 282 -> 91 us against the trace on one CTA).  The
-    // CTAs of the trace take at least RT_MIN_PIX pixels, and no more of them than
-    // fill the device twice
+    // CTAs of the trace take at least RT_MIN_PIX pixels, and there are no more of them
+    // than the device holds at once (16 of 128 threads an SM).  Decided on the call's
+    // largest problem: where its rays do not fit, all candidates take the forms below
     const size_t place_smem = sizeof(int) * (size_t)(max_cells + max_rays);
     if (place_smem <= (size_t)ctx->max_smem - 2048 && n_cand <= 65535) {
         constexpr long long RT_MIN_PIX = 32;

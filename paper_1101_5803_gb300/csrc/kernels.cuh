@@ -476,12 +476,6 @@ __global__ void __launch_bounds__(RT_THREADS) k_rt_rays(const Prob<T>* __restric
         rt_trace_pixels(P, L, cs, c, j0, min(j0 + chunk, P.npix), (int*)nullptr, (int*)nullptr);
 }
 
-// shared memory of k_rt_cells: cell starts, then ray numbers
-template <typename T>
-__host__ inline size_t rt_cells_smem(const Prob<T>& P) {
-    return sizeof(int) * ((size_t)P.ncells + (size_t)P.nrays);
-}
-
 template <typename T>
 __global__ void __launch_bounds__(RT_PLACE_THREADS) k_rt_cells(const Prob<T>* __restrict__ probs,
                                                                const int* __restrict__ cand_prob,
