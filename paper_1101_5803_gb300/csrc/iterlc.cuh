@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(NTHREADS) k_cgls_iter(IterArgs<T> A) {
                 }
             }
             __syncthreads();
-            conv_pass<double, K, false>(w.P2, taps + g.K * g.kp, nullptr, w.qimg, g, CONV_RAW);
+            conv_direct<double, K, false>(w.P2, taps + g.K * g.kp, nullptr, w.qimg, g, CONV_RAW);
             __syncthreads();
             double ss = 0.0;
             for (int i = tid; i < g.ns; i += bs) {
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(NTHREADS) k_cgls_iter(IterArgs<T> A) {
         auto apply_A = [&](const double* v) -> double {
             apply_L<double, double, double, double>(g, w.E, w.inv, v, w.P1);
             __syncthreads();
-            const double ss = conv_pass<double, K, false>(w.P1, taps, w.swp, w.qimg, g, CONV_Q);
+            const double ss = conv_direct<double, K, false>(w.P1, taps, w.swp, w.qimg, g, CONV_Q);
             __syncthreads();
             return ss;
         };

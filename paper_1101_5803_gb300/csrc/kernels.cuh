@@ -1211,9 +1211,9 @@ __device__ __forceinline__ bool conv_by_rows(const Geo<T>& g) {
 
 // conv_pass by rows
 template <int K>
-__device__ __noinline__ double conv_rows_pass(const double* __restrict__ src, const double* __restrict__ taps,
-                                              const double* __restrict__ swp, double* __restrict__ dst, Geo<double> g,
-                                              int mode) {
+__device__ __forceinline__ double conv_rows(const double* __restrict__ src, const double* __restrict__ taps,
+                                            const double* __restrict__ swp, double* __restrict__ dst, const Geo<double>& g,
+                                            int mode) {
     double ss = 0;
     const int kk = K > 0 ? K : g.K, kp = K > 0 ? (K + 3) & ~3 : g.kp;
     for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
@@ -1239,6 +1239,13 @@ __device__ __noinline__ double conv_rows_pass(const double* __restrict__ src, co
     return ss;
 }
 
+template <int K>
+__device__ __noinline__ double conv_rows_pass(const double* __restrict__ src, const double* __restrict__ taps,
+                                              const double* __restrict__ swp, double* __restrict__ dst, Geo<double> g,
+                                              int mode) {
+    return conv_rows<K>(src, taps, swp, dst, g, mode);
+}
+
 // One convolution over all owned tiles (one non-inlined copy of the
 // unrolled tile code per kernel):
 //   CONV_Q   : dst = sqrt(W) * conv, returns sum dst^2
@@ -1246,6 +1253,8 @@ __device__ __noinline__ double conv_rows_pass(const double* __restrict__ src, co
 template <typename T, int K, bool SH>
 __device__ __noinline__ T conv_pass(const T* __restrict__ src, const T* __restrict__ taps,
                                          const T* __restrict__ swp, T* __restrict__ dst, Geo<T> g, int mode) {
+    if constexpr (sizeof(T) == 8 && K > 0)
+        if (conv_by_rows(g)) return conv_rows<K>(src, taps, swp, dst, g, mode);
     T ss = 0;
     for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
         const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
@@ -1276,20 +1285,66 @@ __device__ __noinline__ T conv_pass(const T* __restrict__ src, const T* __restri
     return ss;
 }
 
-// the direct convolution of an image, by rows or by tiles (each a function of
-// its own: with both in one, FP64 images of more than 128 tiles lost 1% to the
-// rows' registers)
+// the direct convolution of an image, by rows or by tiles.  With the taps looped
+// over at run time each is a function of its own: with both in one, images of
+// more than 128 tiles lose 1.2% to the rows' registers (45 x 43, K = 9, 160
+// candidates: 231.9 and 234.9 ms).  With K compiled it is the other way round:
+// the two in one function, 64 tiles at K = 5 take 50.8 ms, apart 51.5
 template <typename T, int K, bool SH>
 __device__ __forceinline__ T conv_direct(const T* src, const T* taps, const T* swp, T* dst, const Geo<T>& g, int mode) {
-    if constexpr (sizeof(T) == 8)
+    if constexpr (sizeof(T) == 8 && K == 0)
         if (conv_by_rows(g)) return conv_rows_pass<K>(src, taps, swp, dst, g, mode);
     return conv_pass<T, K, SH>(src, taps, swp, dst, g, mode);
+}
+
+// conv64_pass by rows (Pc holds the residuals until their sum is taken)
+template <typename T>
+__device__ __forceinline__ double conv64_rows(const Work<T>& w, const Geo<T>& g, int mode) {
+    double ss = 0;
+    const double* src = mode == 0 ? w.Pa : w.Pb;
+    const double* taps = w.taps64 + (mode == 0 ? 0 : g.K * g.kp);
+    for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
+        const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
+        double acc[TILE];
+        conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, g.K, g.kp, acc);
+        const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
+#pragma unroll
+        for (int c = 0; c < TILE; ++c) {
+            if (mode == 0) {
+                const double sw = w.swp[pp + c];
+                const double res = sw * (w.dpad[pp + c] - acc[c]);
+                w.rimg[pp + c] = res;
+                w.Pb[pp + c] = sw * res;
+                w.Pc[pp + c] = res;
+            } else {
+                w.Pc[pp + c] = acc[c];
+            }
+        }
+    }
+    if (mode == 0) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
+            const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
+#pragma unroll
+            for (int r = 0; r < TILE; ++r) {
+                const V4<double> o = ld4(w.Pc + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) ss += o.v[c] * o.v[c];
+            }
+        }
+        __syncthreads();
+    }
+    return ss;
+}
+template <typename T>
+__device__ __noinline__ double conv64_rows_pass(const Work<T> w, Geo<T> g, int mode) {
+    return conv64_rows<T>(w, g, mode);
 }
 
 // FP64 convolution pass of the refinement:
 //   mode 0: res = sqrt(W)(d - conv(Pa)); rimg = (T)res; Pb = sqrt(W) res; returns sum res^2
 //   mode 1: Pc = conv(Pb)
-template <typename T>
+template <typename T, int K>
 __device__ __noinline__ double conv64_pass(const Work<T> w, Geo<T> g, int mode) {
     double ss = 0;
     if (w.fft) {  // the same passes through the FFT convolution
@@ -1310,6 +1365,8 @@ __device__ __noinline__ double conv64_pass(const Work<T> w, Geo<T> g, int mode) 
         fft_convolve<double>(w.fft->d, load, g.ny, store, g.ny, g.nx, mode != 0);
         return ss;
     }
+    if constexpr (sizeof(T) == 8 && K > 0)
+        if (conv_by_rows(g)) return conv64_rows<T>(w, g, mode);
     const double* src = mode == 0 ? w.Pa : w.Pb;
     const double* taps = w.taps64 + (mode == 0 ? 0 : g.K * g.kp);
     for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
@@ -1453,46 +1510,6 @@ __device__ __noinline__ double conv64_df_gen(const double* __restrict__ src, flo
     return ss;
 }
 
-// conv64_pass by rows (Pc holds the residuals until their sum is taken)
-template <typename T>
-__device__ __noinline__ double conv64_rows_pass(const Work<T> w, Geo<T> g, int mode) {
-    double ss = 0;
-    const double* src = mode == 0 ? w.Pa : w.Pb;
-    const double* taps = w.taps64 + (mode == 0 ? 0 : g.K * g.kp);
-    for (int u = threadIdx.x; u < g.ntiles * TILE; u += blockDim.x) {
-        const int y = u / g.tiles_x, tx = u - y * g.tiles_x;
-        double acc[TILE];
-        conv_row64(src + y * g.Wp + tx * TILE + g.sh, g.Wp, taps, g.K, g.kp, acc);
-        const int pp = (y + g.hk) * g.Wp + tx * TILE + g.xoff;
-#pragma unroll
-        for (int c = 0; c < TILE; ++c) {
-            if (mode == 0) {
-                const double sw = w.swp[pp + c];
-                const double res = sw * (w.dpad[pp + c] - acc[c]);
-                w.rimg[pp + c] = res;
-                w.Pb[pp + c] = sw * res;
-                w.Pc[pp + c] = res;
-            } else {
-                w.Pc[pp + c] = acc[c];
-            }
-        }
-    }
-    if (mode == 0) {
-        __syncthreads();
-        for (int t = threadIdx.x; t < g.ntiles; t += blockDim.x) {
-            const int ty = t / g.tiles_x, tx = t - ty * g.tiles_x;
-#pragma unroll
-            for (int r = 0; r < TILE; ++r) {
-                const V4<double> o = ld4(w.Pc + (ty * TILE + r + g.hk) * g.Wp + tx * TILE + g.xoff);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) ss += o.v[c] * o.v[c];
-            }
-        }
-        __syncthreads();
-    }
-    return ss;
-}
-
 // the general kernel's refinement passes: double-float for direct
 // convolution in FP32 contexts, conv64_pass otherwise (FP64 contexts, FFT)
 template <typename T, int KT>
@@ -1503,9 +1520,9 @@ struct Conv64Gen {
                 return conv64_df_gen<KT>(mode == 0 ? w.Pa : w.Pb, w.P1, w.P2, w.taps + (mode == 0 ? 0 : g.K * g.kp),
                                          w.swp, w.dpad, w.rimg, w.Pb, w.Pc, g, mode);
         }
-        if constexpr (sizeof(T) == 8)
+        if constexpr (sizeof(T) == 8 && KT == 0)  // (see conv_direct)
             if (!w.fft && conv_by_rows(g)) return conv64_rows_pass<T>(w, g, mode);
-        return conv64_pass<T>(w, g, mode);
+        return conv64_pass<T, KT>(w, g, mode);
     }
 };
 
