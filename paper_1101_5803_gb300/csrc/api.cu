@@ -991,7 +991,8 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
         return more;
     };
     // Estimated clocks of the classes' items with these forms: the longest item (1.15
-    // of the mean over candidates, up to 2 where problems differ), or the work on all SMs, and
+    // of the mean over candidates, up to 2 where problems differ, 2 in chains, which hold
+    // several lambdas), or the work on all SMs, and
     // part of the other one, since the end of a call is never packed full.  How iteration
     // counts fall with lambda depends on the grid's values, which are device data: the
     // estimate is the geometric mean over counts that fall by 10^0.8 and by 10^2 from
@@ -1016,7 +1017,7 @@ int eval_impl(mirage_ctx* ctx, const mirage_problem_t* probs, int n_probs, const
                 }
             }
             const double full = 0.5 * std::min(1.0, sum / busy);  // its part beside others
-            const double longest = ((1.0 - full) * alone + full * busy) * (1.15 + 0.85 * unlike);
+            const double longest = ((1.0 - full) * alone + full * busy) * (chains ? 2.0 : 1.15 + 0.85 * unlike);
             e += 0.5 * std::log(std::max(sum, longest) + 0.3 * std::min(sum, longest));
             call_time = std::max(sum, longest);
         }

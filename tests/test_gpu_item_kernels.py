@@ -106,3 +106,10 @@ def test_groups_side_by_side_or_in_turn(n):
         for key in KEYS:
             assert torch.equal(a[key][i::4], one[key]), key
     ctx.close()
+
+
+def test_short_chained_calls_run_on_wide_clusters():
+    # a chain holds several lambdas: 12 candidates at 128 x 128 take 175 ms on clusters
+    # of four, where their items one by one would go, and 115 on clusters of eight
+    k = _kernels([(128, 128, 48, 48, 11)], 12, 16, lam_start=np.full(12, 8, np.int32))
+    assert k["cluster8"] == 192, k
